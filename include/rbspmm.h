@@ -360,7 +360,9 @@ typedef struct {
                             every true residual and of the final x (zero-mean solution) */
   int32_t check_every;   /* iterations between host convergence checks (>= 1) */
   int32_t persistent;    /* mixed only: 1 runs each sweep's inner iterations in one cooperative
-                            launch (grid-wide barriers instead of kernel boundaries) */
+                            launch (grid-wide barriers instead of kernel boundaries); 0 lets the
+                            library choose (matrix-free inner operators of moderate size take
+                            that launch too, others two kernels an iteration) */
 } rb_cg_params;
 
 typedef struct {

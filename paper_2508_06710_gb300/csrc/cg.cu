@@ -25,6 +25,7 @@
 #include "reduce.cuh"
 #include "spmm_impl.cuh"
 #include "stencil7.cuh"
+#include "unit7.cuh"
 
 namespace rb {
 
@@ -1075,6 +1076,8 @@ rb_status read_state(const Solver& S_, HostState& h) {
 
 // one sweep's inner iterations of a single system in one cooperative launch (defined below)
 rb_status persistent_inner(Solver& S_, const rb_cg_params& prm, const Layout& L, char* base);
+// whether that launch is the faster way to run them (the default then takes it too)
+bool prefer_persistent(const Solver& S_);
 
 template <int VEC>
 rb_status solve_vec(Solver& S_, const rb_cg_params& prm, const double* B, int64_t ldb, double* X, int64_t ldx,
@@ -1130,6 +1133,7 @@ rb_status solve_vec(Solver& S_, const rb_cg_params& prm, const double* B, int64_
     k_init_outer<<<1, K, 0, S_.s>>>(S_.sc, k);
     int total_inner = 0;
     int sweep = 0;
+    bool one_launch = prm.persistent || prefer_persistent(S_);
     ChunkGraph graph;
     int uses = 0;
     for (;; ++sweep) {
@@ -1146,24 +1150,40 @@ rb_status solve_vec(Solver& S_, const rb_cg_params& prm, const double* B, int64_
       k_ir_init<VEC><<<S_.vg(&k_ir_init<VEC>), kThreads, 0, S_.s>>>(c, r64, r32, p32, d32, dinv32, S_.sc, S_.partials);
       RB_CUDA(cudaGetLastError());
       int it = 0;
-      if (prm.persistent) {
+      if (one_launch) {
         // all of this sweep's inner iterations in one cooperative launch
         rb_cg_params p2 = prm;
         p2.max_iter = prm.max_iter - total_inner;
-        RB_TRY(persistent_inner(S_, p2, L, base));
+        const rb_status launched = persistent_inner(S_, p2, L, base);
+        if (launched != RB_OK) {
+          if (prm.persistent) return launched;
+          // not the caller's choice, and refused (fewer SMs than the device reports): launch by launch
+          cudaGetLastError();
+          clear_error();
+          one_launch = false;
+        }
+      }
+      if (one_launch) {
         unsigned pb[2] = {0, 0};  // pbar[2]: barrier error word, pbar[3]: iterations done
         RB_CUDA(cudaMemcpyAsync(pb, &S_.sc->pbar[2], 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, S_.s));
         RB_CUDA(cudaStreamSynchronize(S_.s));
         ++syncs;
         const unsigned err = pb[0], done = pb[1];
-        if (err) {
+        if (err && prm.persistent) {
           set_error("rb_cg_solve: a grid barrier wait of the persistent inner solve gave up");
           return RB_ETIMEOUT;
+        }
+        if (err) {
+          // not the caller's choice: the sweep is dropped (X is untouched) and the solve goes on
+          // launch by launch, from a fresh direction (scale 0: k_ir_init keeps none)
+          one_launch = false;
+          RB_CUDA(cudaMemsetAsync(S_.sc->oscale, 0, sizeof(S_.sc->oscale), S_.s));
+          continue;
         }
         it = (int)done;
         spmms += it;
       }
-      while (!prm.persistent) {
+      while (!one_launch) {
         RB_TRY(read_state(S_, h));
         ++syncs;
         if (h.n_active == 0 || total_inner + it >= prm.max_iter) break;
@@ -1237,6 +1257,10 @@ struct PSys {
   int n, k, vec, kp;
   int blk0, nblk;  // blocks [blk0, blk0 + nblk) work on this system
   int col0;        // first column of this system in the batch numbering
+  // the unit kernel (k_pcg_units): V floats a unit, each block's share of the system's units, and
+  // how many of them keep r, q and d in shared memory (the rest in the arrays above)
+  Unit7 u7;
+  int uw, uchunk, cap_r, cap_q, cap_d;
 };
 
 struct PBatch {
@@ -1576,6 +1600,375 @@ __global__ void __launch_bounds__(kPThreads) k_pcg_batch(PBatch b) {
   if (lead && threadIdx.x == 0) recount(b.sys[my].sc, b.sys[my].k);
 }
 
+// ---------------------------------------------------------- the same, on units (unit7.cuh)
+// The persistent solve of systems whose inner operators are all matrix-free.  Each block owns a
+// contiguous range of a system's units for the whole launch, so the vectors that only their
+// owner touches (r, then q, then d, as far as they fit) stay in its shared memory and do not move.
+// One block of 768 threads per SM (a multiple of 3 and 256: a thread's columns are the same in
+// every unit it visits, so its sums and its alpha and beta are per float; 960 threads of 64
+// registers: 52.3 against 50.2 ms on the batch below).  Channel 192 x 128 x 96, k = 3, per
+// iteration: 52 us (two kernels a step: 77), of which q = A p 21, the update 17, the two barriers
+// 9 and the column sums 5; bound by instruction issue and by L2: 20 M warp instructions (IPC 1.2),
+// 65 MB read and 57 MB written of the vectors that are not in shared memory.  The five uneven
+// systems 64^3 k = 8, 128^3 k = 1, 3 x 96 x 64 x 48 k = 3: 68.3 -> 50.6 ms.  Measured and not kept:
+// p in shared memory instead of r (104 ms on the channel against 82: r and d then move twice), plain
+// loads of p through L1 (97), two to four units' loads issued together (109 to 118: fewer threads).
+constexpr int kUThreads = 768;
+constexpr int kUWarps = kUThreads / 32;
+constexpr int kUGridMax = 256;  // blocks (one per SM)
+
+struct UShared {
+  UnitTab tab;  // the block's system's per-axis tables
+  float red[kUWarps * 2 * 64];
+  double out[2 * K], tot[2 * K];
+  double rz[K], alpha[K], beta[K];
+  int state[K], iters[K], met[K];
+  int go, mine;
+};
+
+// Block sums of the threads' per-float sums t[quantity][float]: column of float e is
+// (rem + e) mod KC (KC in 1..3), or rem + e (KC = 0, kp chunks per row in adjacent lanes)
+template <int KC, int V>
+__device__ __forceinline__ void ublock_reduce(float (&t)[2][V], int rem, int k, UShared& sh) {
+  constexpr int N = KC == 0 ? V : KC;
+  float s[2][N];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+#pragma unroll
+    for (int c = 0; c < N; ++c) s[q][c] = KC == 0 ? t[q][c % V] : 0.0f;
+    if constexpr (KC != 0) {
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        const int col = (rem + e) % KC;
+#pragma unroll
+        for (int c = 0; c < N; ++c) s[q][c] += col == c ? t[q][e] : 0.0f;
+      }
+    }
+  }
+  const int kp = KC == 0 ? k / V : 1;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) warp_fold<float, N>(s[q], kp);
+  if (lane < kp) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int c = 0; c < N; ++c) sh.red[(w * 2 + q) * 64 + lane * N + c] = s[q][c];
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < 2 * k) {
+    const int q = threadIdx.x / k, j = threadIdx.x % k;
+    double v = 0.0;
+    for (int ww = 0; ww < kUWarps; ++ww) v += (double)sh.red[(ww * 2 + q) * 64 + j];
+    sh.out[threadIdx.x] = v;
+  }
+  __syncthreads();
+}
+
+template <int V>
+__device__ __forceinline__ Vec<float, V> uload(const float* s, const float* g, uint32_t li, uint32_t cap) {
+  if (li < cap) return ldv_rw<float, V>(s + (size_t)li * V);
+  return ldv_cg<float, V>(g);
+}
+template <int V>
+__device__ __forceinline__ void ustore(float* s, float* g, uint32_t li, uint32_t cap, const Vec<float, V>& v) {
+  if (li < cap) stv<float, V>(s + (size_t)li * V, v);
+  else stv<float, V>(g, v);
+}
+
+struct UMem {
+  float *r, *q, *d;  // shared memory
+  uint32_t u0, cnt;  // the block's units
+};
+
+template <int KC, int V>
+__device__ __forceinline__ Vec<float, V> udinv(const PSys& S, uint32_t F) {
+  if (!S.dinv) {
+    Vec<float, V> d;
+#pragma unroll
+    for (int e = 0; e < V; ++e) d.v[e] = 1.0f;
+    return d;
+  }
+  const uint32_t cell0 = unit7_cell<KC>(S.u7, F);
+  return unit7_cells<KC, V>(S.dinv, cell0, (int)(F - cell0 * (uint32_t)S.k));
+}
+
+// phase A: q = A p with p . q and q . D^-1 q (t[0], t[1] per float)
+template <int KC, int V>
+__device__ __forceinline__ void uphase_q(const PSys& S, const UMem& m, UShared& sh) {
+  float t[2][V];
+#pragma unroll
+  for (int e = 0; e < V; ++e) t[0][e] = t[1][e] = 0.0f;
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t w0 = threadIdx.x - lane; w0 < m.cnt; w0 += kUThreads) {  // whole warps
+    const int last = (int)min(31u, m.cnt - 1 - w0);  // the warp's last lane with a unit
+    const uint32_t li = min(w0 + lane, m.cnt - 1);
+    const UnitPos u = unit7_pos(S.u7, (m.u0 + li) * V);
+    const Vec<float, V> d = udinv<KC, V>(S, u.F);
+    Vec<float, V> x0, q;
+    unit7_apply<KC, V>(S.u7, sh.tab, S.p, u, last, x0, q);
+    if ((int)lane <= last) {
+      ustore<V>(m.q, S.q + u.F, li, S.cap_q, q);
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        t[0][e] = fmaf(x0.v[e], q.v[e], t[0][e]);
+        t[1][e] = fmaf(q.v[e], d.v[e] * q.v[e], t[1][e]);
+      }
+    }
+  }
+  const int rem0 = (int)(((m.u0 + threadIdx.x) * (uint32_t)V) % (uint32_t)S.k);
+  ublock_reduce<KC, V>(t, rem0, S.k, sh);
+}
+
+// phase B: d += alpha p, r -= alpha q, p = D^-1 r + beta p on active columns; r . D^-1 r, r . r
+template <int KC, int V>
+__device__ __forceinline__ void uphase_xrp(const PSys& S, const UMem& m, UShared& sh) {
+  float t[2][V], al[V], be[V];
+  bool on[V];
+  const int rem0 = (int)(((m.u0 + threadIdx.x) * (uint32_t)V) % (uint32_t)S.k);
+#pragma unroll
+  for (int e = 0; e < V; ++e) {
+    const int j = KC == 0 ? rem0 + e : (rem0 + e) % (KC ? KC : 1);
+    on[e] = sh.state[j] == ST_ACTIVE;
+    al[e] = on[e] ? (float)sh.alpha[j] : 0.f;
+    be[e] = on[e] ? (float)sh.beta[j] : 0.f;
+    t[0][e] = t[1][e] = 0.0f;
+  }
+  for (uint32_t li = threadIdx.x; li < m.cnt; li += kUThreads) {
+    const uint32_t F = (m.u0 + li) * V;
+    Vec<float, V> pv = ldv_cg<float, V>(S.p + F);
+    Vec<float, V> xv = uload<V>(m.d, S.d + F, li, S.cap_d);
+    Vec<float, V> rv = uload<V>(m.r, S.r + F, li, S.cap_r);
+    const Vec<float, V> qv = uload<V>(m.q, S.q + F, li, S.cap_q);
+    const Vec<float, V> d = udinv<KC, V>(S, F);
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+      xv.v[e] = fmaf(al[e], pv.v[e], xv.v[e]);
+      rv.v[e] = fmaf(-al[e], qv.v[e], rv.v[e]);
+      const float zz = d.v[e] * rv.v[e];
+      pv.v[e] = on[e] ? fmaf(be[e], pv.v[e], zz) : pv.v[e];
+      t[0][e] = fmaf(rv.v[e], zz, t[0][e]);
+      t[1][e] = fmaf(rv.v[e], rv.v[e], t[1][e]);
+    }
+    stv<float, V>(S.p + F, pv);
+    ustore<V>(m.d, S.d + F, li, S.cap_d, xv);
+    ustore<V>(m.r, S.r + F, li, S.cap_r, rv);
+  }
+  ublock_reduce<KC, V>(t, rem0, S.k, sh);
+}
+
+// the shared-memory parts of r and d from (or back to) their arrays
+template <int V>
+__device__ __forceinline__ void umove(const PSys& S, const UMem& m, bool in) {
+  for (uint32_t li = threadIdx.x; li < m.cnt; li += kUThreads) {
+    const uint32_t F = (m.u0 + li) * V;
+    if (li < (uint32_t)S.cap_r) {
+      if (in) stv<float, V>(m.r + (size_t)li * V, ldv_cg<float, V>(S.r + F));
+      else stv<float, V>(S.r + F, ldv_rw<float, V>(m.r + (size_t)li * V));
+    }
+    if (li < (uint32_t)S.cap_d) {
+      if (in) stv<float, V>(m.d + (size_t)li * V, ldv_cg<float, V>(S.d + F));
+      else stv<float, V>(S.d + F, ldv_rw<float, V>(m.d + (size_t)li * V));
+    }
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ int unit_case(const PSys& S) {
+  return S.k % 4 == 0 ? 0 : (S.k - 1) * 3 + (S.uw == 4 ? 3 : S.uw);  // 1..9: k = 1..3, width 1, 2, 4
+}
+
+#define RB_UNIT_SWITCH(S, CALL)          \
+  switch (unit_case(S)) {                \
+    case 0: CALL(0, 4); break;           \
+    case 1: CALL(1, 1); break;           \
+    case 2: CALL(1, 2); break;           \
+    case 3: CALL(1, 4); break;           \
+    case 5: CALL(2, 2); break;           \
+    case 6: CALL(2, 4); break;           \
+    case 7: CALL(3, 1); break;           \
+    case 8: CALL(3, 2); break;           \
+    case 9: CALL(3, 4); break;           \
+  }
+#define RB_WIDTH_SWITCH(S, CALL) \
+  switch (S.uw) {                \
+    case 1: CALL(1); break;      \
+    case 2: CALL(2); break;      \
+    case 4: CALL(4); break;      \
+  }
+
+// Grid-wide barrier: one counter that only grows (zeroed before the launch), `phase` barriers
+// passed before this one.  One release-add per block and one acquire-polled word: the fences of
+// grid_barrier and its second counter cost about a microsecond a barrier more.  Bounded as there.
+__device__ bool unit_barrier(const PBatch& b, unsigned phase, UShared& sh) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    const unsigned target = (phase + 1u) * (gridDim.x + (unsigned)b.extra_arrivals);
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(b.bar), "r"(1u) : "memory");
+    const unsigned long long t0 = globaltimer_ns();
+    unsigned seen;
+    for (unsigned n = 1;; ++n) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(b.bar) : "memory");
+      if ((int)(seen - target) >= 0) break;
+      if (n % 64 == 0) {
+        if (*(volatile int*)b.err) {
+          ok = 0;
+          break;
+        }
+        if (globaltimer_ns() - t0 > b.timeout_ns) {
+          atomicCAS(b.err, 0, 1);
+          ok = 0;
+          break;
+        }
+      }
+    }
+    sh.go = ok;
+  }
+  __syncthreads();
+  return sh.go != 0;
+}
+
+// a block's partial of quantity q, batch column c: the blocks' values of one sum lie together
+__device__ __forceinline__ size_t upartial(int q, int c, int block) { return ((size_t)q * K + c) * kUGridMax + block; }
+
+// psys_totals of this kernel's block size and layout
+__device__ __forceinline__ void usys_totals(const PBatch& b, const PSys& S, int q0, int nq, double* out) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = w; i < nq; i += kUWarps) {
+    const int q = q0 + i / S.k, c = S.col0 + i % S.k;
+    double s = 0.0;
+    for (int bb = lane; bb < S.nblk; bb += 32) s += __ldcg(&b.partials[upartial(q, c, S.blk0 + bb)]);
+    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) out[i] = s;
+  }
+  __syncthreads();
+}
+
+// The control flow of k_pcg_batch (see there) around the unit phases
+// (ONE: a single system, whose fields are then operands at fixed places of the parameter bank
+// instead of indexed loads)
+template <bool ONE>
+__global__ void __launch_bounds__(kUThreads, 1) k_pcg_units(const __grid_constant__ PBatch b) {
+  extern __shared__ __align__(16) float ubuf[];
+  __shared__ UShared sh;
+  int my = 0;
+  if constexpr (!ONE)
+    for (int s = 0; s < b.n_sys; ++s)
+      if ((int)blockIdx.x >= b.sys[s].blk0 && (int)blockIdx.x < b.sys[s].blk0 + b.sys[s].nblk) my = s;
+  const PSys& S = b.sys[ONE ? 0 : my];  // every block has a system
+  const bool lead = (int)blockIdx.x == S.blk0;
+  const int j = threadIdx.x;
+  if (j < S.k) {
+    sh.state[j] = __ldcg(&S.sc->state[j]);
+    sh.rz[j] = __ldcg(&S.sc->rz[j]);
+    sh.iters[j] = __ldcg(&S.sc->iters[j]);
+    sh.met[j] = 0;
+  }
+  UMem m;
+  const uint32_t units = (uint32_t)(((int64_t)S.n * S.k) / S.uw);
+  m.u0 = min((uint32_t)(blockIdx.x - S.blk0) * (uint32_t)S.uchunk, units);
+  m.cnt = min((uint32_t)S.uchunk, units - m.u0);
+  m.r = ubuf;
+  m.q = m.r + (size_t)S.cap_r * S.uw;
+  m.d = m.q + (size_t)S.cap_q * S.uw;
+  const int entry_go = pany_active(b) ? 1 : 0;
+  unit7_table(S.u7, sh.tab);
+#define RB_U_IN(V) umove<V>(S, m, true)
+  RB_WIDTH_SWITCH(S, RB_U_IN)
+#undef RB_U_IN
+  for (int it = 0; it < b.max_iter; ++it) {
+    if (j == 0) {
+      int g = entry_go;
+      if (it >= 2) {
+        g = 0;
+        for (int s = 0; s < b.n_sys; ++s) g |= __ldcg(&b.sys[s].sc->pact[it & 1]);
+      }
+      sh.go = g;
+      int a = 0;
+      for (int c = 0; c < S.k; ++c) a |= sh.state[c] == ST_ACTIVE;
+      sh.mine = a;
+    }
+    __syncthreads();
+    if (!sh.go) break;
+    const bool mine = sh.mine != 0;
+    if (lead && mine && j == 0) atomicMax(b.bar + 3, (unsigned)(it + 1));  // iterations with work
+    if (mine) {
+#define RB_U_Q(KC, V) uphase_q<KC, V>(S, m, sh)
+      RB_UNIT_SWITCH(S, RB_U_Q)
+#undef RB_U_Q
+      if (j < 2 * S.k) b.partials[upartial(j / S.k, S.col0 + j % S.k, blockIdx.x)] = sh.out[j];
+    }
+    if (!unit_barrier(b, 2u * it, sh)) return;
+    if (mine) {
+      usys_totals(b, S, 0, 2 * S.k, sh.tot);
+      if (j < S.k) {
+        const double pq = sh.tot[j], qdq = sh.tot[S.k + j];
+        double al = 0.0, be = 0.0;
+        if (sh.state[j] == ST_ACTIVE) {
+          if (!(pq > 0.0) || !isfinite(pq) || !isfinite(qdq)) {
+            sh.state[j] = ST_DONE;
+          } else {
+            const double ipq = 1.0 / pq;
+            al = sh.rz[j] * ipq;
+            const double bb = al * qdq * ipq - 1.0;
+            be = (bb > 0.0 && isfinite(bb)) ? bb : 0.0;
+          }
+        }
+        sh.alpha[j] = al;
+        sh.beta[j] = be;
+        if (lead) S.sc->pq[j] = pq, S.sc->alpha[j] = al, S.sc->beta[j] = be;
+      }
+      __syncthreads();
+#define RB_U_X(KC, V) uphase_xrp<KC, V>(S, m, sh)
+      RB_UNIT_SWITCH(S, RB_U_X)
+#undef RB_U_X
+      if (j < 2 * S.k) b.partials[upartial(2 + j / S.k, S.col0 + j % S.k, blockIdx.x)] = sh.out[j];
+    }
+    if (!unit_barrier(b, 2u * it + 1u, sh)) return;
+    if (mine) {
+      usys_totals(b, S, 2, 2 * S.k, sh.tot);
+      if (j < S.k) {
+        const double rz_new = sh.tot[j], rr_new = sh.tot[S.k + j];
+        if (sh.state[j] == ST_ACTIVE) {
+          sh.iters[j] += 1;
+          sh.rz[j] = rz_new;
+          if (!isfinite(rr_new) || !isfinite(rz_new)) sh.state[j] = ST_DONE;
+          else if (rr_new <= S.sc->tol2[j]) sh.met[j] = 1;
+          if (lead) S.sc->rr[j] = rr_new;
+        }
+      }
+      __syncthreads();
+      if (j == 0) {
+        bool all = true;
+        for (int c = 0; c < S.k; ++c) all &= sh.state[c] != ST_ACTIVE || sh.met[c] != 0;
+        if (all)
+          for (int c = 0; c < S.k; ++c)
+            if (sh.state[c] == ST_ACTIVE) sh.state[c] = ST_DONE;
+      }
+      __syncthreads();
+      if (lead && j < S.k) {
+        S.sc->iters[j] = sh.iters[j];
+        S.sc->state[j] = sh.state[j];
+        S.sc->rz[j] = sh.rz[j];
+      }
+      __syncthreads();
+      if (lead && j == 0) recount(S.sc, S.k);
+    }
+    if (lead && j == 0) {
+      int a = 0;
+      for (int c = 0; c < S.k; ++c) a |= sh.state[c] == ST_ACTIVE;
+      S.sc->pact[it & 1] = a;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+#define RB_U_OUT(V) umove<V>(S, m, false)
+  RB_WIDTH_SWITCH(S, RB_U_OUT)
+#undef RB_U_OUT
+  if (lead && j == 0) recount(S.sc, S.k);
+}
+
 // ------------------------------------------------------------------ host side of the batch
 
 int sm_count() {
@@ -1603,14 +1996,15 @@ int pcg_blocks_per_sm() {
 
 constexpr int kPGridMax = 152 * 4;  // partials capacity: 4 resident blocks of 512 threads per SM
 
-// Blocks per system in proportion to the bytes one iteration streams (rows x (2 + k)), at
-// least one each; the first total_cols blocks double as the column reducers.
-void partition_blocks(PBatch& pb, int grid) {
+// Blocks per system in proportion to the bytes one iteration streams (rows x (2 + k); the unit
+// kernel's: rows x k), at least one each.
+void partition_blocks(PBatch& pb, int grid, bool units) {
+  const int extra = units ? 0 : 2;
   double W = 0.0;
-  for (int s = 0; s < pb.n_sys; ++s) W += (double)pb.sys[s].n * (2 + pb.sys[s].k);
+  for (int s = 0; s < pb.n_sys; ++s) W += (double)pb.sys[s].n * (extra + pb.sys[s].k);
   int used = 0;
   for (int s = 0; s < pb.n_sys; ++s) {
-    int nb = (int)std::floor(grid * ((double)pb.sys[s].n * (2 + pb.sys[s].k)) / std::max(W, 1.0));
+    int nb = (int)std::floor(grid * ((double)pb.sys[s].n * (extra + pb.sys[s].k)) / std::max(W, 1.0));
     nb = std::max(1, nb);
     pb.sys[s].nblk = nb;
     used += nb;
@@ -1626,7 +2020,7 @@ void partition_blocks(PBatch& pb, int grid) {
     int best = 0;
     double wb = -1.0;
     for (int s = 0; s < pb.n_sys; ++s) {
-      const double w = (double)pb.sys[s].n * (2 + pb.sys[s].k) / pb.sys[s].nblk;
+      const double w = (double)pb.sys[s].n * (extra + pb.sys[s].k) / pb.sys[s].nblk;
       if (w > wb) wb = w, best = s;
     }
     ++pb.sys[best].nblk;
@@ -1639,18 +2033,50 @@ void partition_blocks(PBatch& pb, int grid) {
   }
 }
 
-rb_status launch_pcg(const PBatch& pb, int grid, cudaStream_t s) {
+// Shared memory of k_pcg_units a block may use beside its static part (one block per SM)
+constexpr size_t kUSmem = 188 * 1024;
+
+// Whether every system takes the unit kernel; then fills their unit fields for `grid` blocks
+// (the partition must be made)
+bool units_ok(const PBatch& pb) {
+  for (int i = 0; i < pb.n_sys; ++i)
+    if (!pb.sys[i].mf || !unit7_table_fits(pb.sys[i].st.n) || unit7_width(pb.sys[i].st.n, pb.sys[i].k) == 0 ||
+        pb.sys[i].n == 0)
+      return false;
+  return pb.n_sys > 0;
+}
+
+void fill_units(PBatch& pb) {
+  for (int i = 0; i < pb.n_sys; ++i) {
+    PSys& S = pb.sys[i];
+    S.uw = unit7_width(S.st.n, S.k);
+    S.u7.init(S.st, S.k);
+    const int64_t units = ((int64_t)S.n * S.k) / S.uw;
+    // ranges start at multiples of 64 units: a row's chunks (k = 4 kp) stay in adjacent lanes
+    S.uchunk = (int)(((units + S.nblk - 1) / S.nblk + 63) / 64 * 64);
+    int64_t left = (int64_t)(kUSmem / (4 * S.uw)) / 64 * 64;
+    for (int* cap : {&S.cap_r, &S.cap_q, &S.cap_d}) {
+      *cap = (int)std::min<int64_t>(left, S.uchunk);
+      left -= *cap;
+    }
+  }
+}
+
+rb_status launch_pcg(const PBatch& pb, int grid, bool units, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
+  auto* unit_kernel = pb.n_sys == 1 ? &k_pcg_units<true> : &k_pcg_units<false>;
+  if (units) RB_TRY(opt_in_smem(reinterpret_cast<const void*>(unit_kernel), kUSmem));
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kPThreads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.blockDim = dim3(units ? kUThreads : kPThreads);
+  cfg.dynamicSmemBytes = units ? kUSmem : 0;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  RB_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_batch, pb));
+  if (units) RB_CUDA(cudaLaunchKernelEx(&cfg, unit_kernel, pb));
+  else RB_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_batch, pb));
   return RB_OK;
 }
 
@@ -1797,6 +2223,17 @@ void solve_tail(Solver& S_, const rb_cg_params& prm, const double* B, int64_t ld
     default: CALL(1); break;     \
   }
 
+// Up to 10 M floats per vector, of which the blocks' shared memory holds 7.3 M (one of the
+// vectors entirely, on most grids).  Measured per iteration, one launch against two kernels a
+// step: channel 192 x 128 x 96 k = 3 (7.1 M) 52 / 77 us, 128^3 k = 4 (8.4 M) 67 / 86, 128^3 k = 1
+// 25 / 33, 45 x 64 x 31 k = 1 (one float a unit) 16 / 19, 32^3 k = 1 21 / 27; beyond, the vectors
+// stream from HBM either way and one block per SM keeps fewer loads in flight: 192 x 192 x 160
+// k = 3 (17.7 M) 164 / 160, the channel at k = 16 (37.7 M) 343 / 286.
+bool prefer_persistent(const Solver& S_) {
+  return S_.A32->format == RB_STENCIL && unit7_table_fits(S_.A32->st_n) && unit7_width(S_.A32->st_n, S_.k) != 0 &&
+         S_.n * S_.k <= 10000000;
+}
+
 rb_status persistent_inner(Solver& S_, const rb_cg_params& prm, const Layout& L, char* base) {
   PBatch pb;
   pb.n_sys = 1;
@@ -1808,10 +2245,12 @@ rb_status persistent_inner(Solver& S_, const rb_cg_params& prm, const Layout& L,
   pb.max_iter = prm.max_iter;
   pb.extra_arrivals = 0;
   pb.timeout_ns = 2000000000ull;
-  const int grid = std::min(kPGridMax, pcg_blocks_per_sm() * sm_count());
-  partition_blocks(pb, grid);
+  const bool units = units_ok(pb);
+  const int grid = units ? std::min(kUGridMax, sm_count()) : std::min(kPGridMax, pcg_blocks_per_sm() * sm_count());
+  partition_blocks(pb, grid, units);
+  if (units) fill_units(pb);
   RB_CUDA(cudaMemsetAsync(S_.sc->pbar, 0, 4 * sizeof(unsigned), S_.s));
-  return launch_pcg(pb, grid, S_.s);
+  return launch_pcg(pb, grid, units, S_.s);
 }
 
 void fill_report(const CgScal& hs, int k, int mixed, rb_cg_report& rep, rb_status& worst) {
@@ -1882,7 +2321,7 @@ rb_status batch_sequence(rb_batch* bt, Solver* SV, PBatch& pb, int grid, const d
 #undef RB_HEAD
     }
     RB_CUDA(cudaMemsetAsync(bt->bar, 0, 4 * sizeof(unsigned), s));
-    RB_TRY(launch_pcg(pb, grid, s));
+    RB_TRY(launch_pcg(pb, grid, units_ok(pb), s));
     for (int i = 0; i < bt->n_sys; ++i) {
       char* base = ws_base(bt->work[i]);
 #define RB_TAIL(V) sweep_tail<V>(SV[i], X[i], ldx[i], bt->L[i], base)
@@ -1918,12 +2357,14 @@ rb_status batch_prepare(rb_batch* bt, Solver* SV, PBatch& pb, int& grid, const d
   pb.max_iter = bt->prm.max_iter;
   pb.extra_arrivals = bt->extra_arrivals;
   pb.timeout_ns = (unsigned long long)(bt->timeout_ms * 1e6);
-  const int cap = pcg_blocks_per_sm();
+  const bool units = units_ok(pb);
+  const int cap = units ? 1 : pcg_blocks_per_sm();
   const int bps = bt->blocks_per_sm > 0 ? std::min(bt->blocks_per_sm, cap) : cap;
-  grid = std::min(kPGridMax, bps * sm_count());
+  grid = std::min(units ? kUGridMax : kPGridMax, bps * sm_count());
   grid = std::max(grid, pb.total_cols);
   RB_REQUIRE(grid <= cap * sm_count(), "batch: %d columns need more co-resident blocks than fit", pb.total_cols);
-  partition_blocks(pb, grid);
+  partition_blocks(pb, grid, units);
+  if (units) fill_units(pb);
   return RB_OK;
 }
 
