@@ -272,6 +272,65 @@ __global__ void __launch_bounds__(kThreads) k_mg_restrict_st(Transfer3<T> tr, in
   }
 }
 
+// The restriction by rows.  P^T is a product of three 1-D maps, so a block takes whole x rows: the y
+// and z maps combine rows of consecutive floats (whatever their cells and columns: every load is
+// contiguous and a thread's 16 loads are independent), the x map then runs on the combined row in
+// shared memory: 2 x 16 fine values per coarse one instead of 4 x 16.  Bound by the latency of one
+// round of loads on the coarse levels (the kernel above waits for four rows' gathers after another
+// four's) and by L2 on the finest.  Channel k = 3, per launch: 192 x 128 x 96 22 -> 14 us,
+// 96 x 64 x 48 and coarser 10 -> 6.2 us.  (The prolongation in the same form was slower, 11 -> 13 us:
+// it has only 8 gathers per cell, all independent.)  rb rows per block, nx k floats a row (V of
+// them per load).
+template <int V>
+__global__ void __launch_bounds__(kThreads) k_mg_restrict_rows(Transfer3<float> tr, int k, int rb, FastDiv dunits,
+                                                                FastDiv dout, FastDiv dk, const float* __restrict__ rf,
+                                                                float* __restrict__ rc, const int* __restrict__ gate) {
+  if (gate && *gate == 0) return;
+  extern __shared__ __align__(16) float srow[];
+  const int nx = tr.nf[0], ny = tr.nf[1], cnx = nx / 2, cny = ny / 2;
+  const int line = nx * k, units = line / V, out = cnx * k;
+  const int row0 = blockIdx.x * rb, rows = min(rb, cny * (tr.nf[2] / 2) - row0);
+  for (int t = threadIdx.x; t < rows * units; t += kThreads) {
+    const int r = (int)dunits.div((uint32_t)t), u = t - r * units;
+    const int row = row0 + r, K3 = row / cny, J = row - K3 * cny;
+    const TAxisTab<float>& ty = tr.ta[1][J];
+    const TAxisTab<float>& tz = tr.ta[2][K3];
+    const int ncy = ty.cnt, ncz = tz.cnt;
+    Vec<float, V> acc;
+#pragma unroll
+    for (int e = 0; e < V; ++e) acc.v[e] = 0.0f;
+    // a coarse cell has 4 fine positions per axis away from a wall: sixteen loads in flight
+    for (int a0 = 0; a0 < ncz; a0 += 4)
+      for (int b0 = 0; b0 < ncy; b0 += 4) {
+        Vec<float, V> v[16];
+#pragma unroll
+        for (int ab = 0; ab < 16; ++ab) {
+          const int a = min(a0 + ab / 4, ncz - 1), b = min(b0 + ab % 4, ncy - 1);
+          v[ab] = ldv<float, V>(rf + (int64_t)(ty.t[b] + ny * tz.t[a]) * line + u * V);
+        }
+#pragma unroll
+        for (int ab = 0; ab < 16; ++ab) {
+          const int a = a0 + ab / 4, b = b0 + ab % 4;
+          const float w = a < ncz && b < ncy ? tz.w[a] * ty.w[b] : 0.0f;
+#pragma unroll
+          for (int e = 0; e < V; ++e)
+            acc.v[e] = a < ncz && b < ncy ? fmaf(w, v[ab].v[e], acc.v[e]) : acc.v[e];
+        }
+      }
+    stv<float, V>(srow + r * line + u * V, acc);
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < rows * out; t += kThreads) {
+    const int r = (int)dout.div((uint32_t)t), o = t - r * out;
+    const int I = (int)dk.div((uint32_t)o), c = o - I * k;
+    const TAxisTab<float>& tx = tr.ta[0][I];
+    const float* s = srow + r * line + c;
+    float y = 0.0f;
+    for (int q = 0; q < tx.cnt; ++q) y = fmaf(tx.w[q], s[tx.t[q] * k], y);
+    rc[(int64_t)(row0 + r) * out + o] = y;
+  }
+}
+
 // ------------------------------------------------------------------- line smoothing
 // Block Jacobi over the grid lines along one wall-bounded axis (the strongly coupled one of a
 // wall-refined grid): the block of a line is the tridiagonal part of A along it (A's diagonal
@@ -1319,6 +1378,9 @@ const T* dinv_of(const rb_op* op) {
   else return op->dinv32;
 }
 
+// row blocks wanted before a block takes more than one row: two per SM
+constexpr int kSpread = 2 * 152;
+
 template <typename T, int VEC>
 struct Cycle {
   const rb_mg* g;
@@ -1361,6 +1423,26 @@ struct Cycle {
       t.init_div();
     }
     return t;
+  }
+
+  // The restriction by rows: V floats per load, as many rows per block as give its threads two
+  // units each, while the rows fit the 48 KB of shared memory that need no opt-in (false: they do not)
+  bool restrict_rows(const rb_mg_level& lv, const float* rf, float* rc) const {
+    if constexpr (sizeof(T) != 4) return false;
+    else {
+      const int line = lv.n[0] * k, v = line % 4 == 0 ? 4 : 2;  // n_x is even where the grid coarsens
+      const int units = line / v, rows = (lv.n[1] / 2) * (lv.n[2] / 2);
+      if ((size_t)line * 4 > 48 * 1024) return false;
+      const int rb = std::max(1, std::min({2 * kThreads / units, 48 * 1024 / (4 * line), (rows + kSpread - 1) / kSpread}));
+      FastDiv du, dout, dk;
+      du.init((uint32_t)units), dout.init((uint32_t)(line / 2)), dk.init((uint32_t)k);
+      auto go = [&](auto* kern) {
+        kern<<<(rows + rb - 1) / rb, kThreads, (size_t)rb * line * 4, s>>>(tr_view(lv), k, rb, du, dout, dk, rf, rc, gate);
+      };
+      if (v == 4) go(&k_mg_restrict_rows<4>);
+      else go(&k_mg_restrict_rows<2>);
+      return true;
+    }
   }
 
   // one product-shaped pass over a level (CSR or matrix-free)
@@ -1420,7 +1502,8 @@ struct Cycle {
     // residual, restriction, the next level, prolongation-add
     sweep<SW_RESID, false>(lv, bufs[c], r, dinv, static_cast<T*>(lv.res), none);
     const rb_mg_level& nx = g->lv[l + 1];
-    if (mf()) {
+    if (mf() && restrict_rows(lv, static_cast<const float*>(lv.res), static_cast<float*>(nx.rhs))) {
+    } else if (mf()) {
       auto* rk = &k_mg_restrict_st<T, VEC>;
       rk<<<grid(rk, nx.cells), kThreads, 0, s>>>(tr_view(lv), nx.cells, k, kp, static_cast<const T*>(lv.res),
                                                 static_cast<T*>(nx.rhs), gate);
