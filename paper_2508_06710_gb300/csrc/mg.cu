@@ -66,6 +66,7 @@ struct MgScal {
   double bb[K], tol2[K], mean[K], scale[K], rr_true[K];
   int ostate[K];
   int n_active, n_oactive;
+  int left;  // iterations a refinement solve may still run (max_iter at its start)
   unsigned counter[8];
 };
 
@@ -737,13 +738,17 @@ __global__ void __launch_bounds__(kThreads) k_mgcg_q(CsrArgs<T> a, Stencil7<T> s
 }
 
 // x += alpha p, r -= alpha q, r . r; the last block counts the iteration and, for a
-// refinement sweep's inner solve (INNER), stops columns whose r . r reached itol2
+// refinement sweep's inner solve (INNER), stops columns whose r . r reached itol2 and tells the
+// sweep's graph (loop, 0 outside one) whether to run another iteration
 template <typename T, int VEC, bool INNER>
 __global__ void __launch_bounds__(kThreads) k_mgcg_xr(int64_t n, int k, int kp, T* __restrict__ x,
                                                        T* __restrict__ r, const T* __restrict__ p,
                                                        const T* __restrict__ q, MgScal* __restrict__ sc,
-                                                       double* __restrict__ partials) {
-  if (sc->n_active == 0) return;
+                                                       double* __restrict__ partials, cudaGraphConditionalHandle loop) {
+  if (sc->n_active == 0) {
+    if (INNER && loop && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(loop, 0);
+    return;
+  }
   __shared__ RedSmem<1> red;
   const int R = kThreads / kp;
   const int chunk = threadIdx.x % kp;
@@ -782,7 +787,13 @@ __global__ void __launch_bounds__(kThreads) k_mgcg_xr(int64_t n, int k, int kp, 
     if (!isfinite(tot)) sc->state[j] = INNER ? MG_DONE : MG_BREAKDOWN;
   }
   __syncthreads();
-  if (threadIdx.x == 0) mg_recount(sc, k);
+  if (threadIdx.x == 0) {
+    mg_recount(sc, k);
+    if constexpr (INNER) {
+      sc->left -= 1;
+      if (loop) cudaGraphSetConditional(loop, sc->n_active > 0 && sc->left > 0 ? 1 : 0);
+    }
+  }
 }
 
 // p = z + beta p (beta = 0 where a column is not iterating); INIT: p = z, whatever p held
@@ -821,7 +832,8 @@ enum ResidKind : int { TR_INIT = 0, TR_CHECK = 1 };
 template <int VEC>
 __global__ void __launch_bounds__(kThreads) k_mg_true_resid(CsrArgs<double> a, const double* __restrict__ b,
                                                              int64_t ldb, double* __restrict__ rt, int kind,
-                                                             int project, double rtol2, MgScal* __restrict__ sc,
+                                                             int project, double rtol2, int max_iter,
+                                                             MgScal* __restrict__ sc,
                                                              double* __restrict__ partials) {
   __shared__ RedSmem<4> red;
   const int R = kThreads / a.kp;
@@ -891,7 +903,10 @@ __global__ void __launch_bounds__(kThreads) k_mg_true_resid(CsrArgs<double> a, c
     if (sc->state[j] == MG_BREAKDOWN) sc->ostate[j] = MG_BREAKDOWN;
   }
   __syncthreads();
-  if (threadIdx.x == 0) mg_recount(sc, a.k);
+  if (threadIdx.x == 0) {
+    if (kind == TR_INIT) sc->left = max_iter;
+    mg_recount(sc, a.k);
+  }
 }
 
 // out = (rt - mean) * inv (per column), in the solve's type T; zero for columns that are not
@@ -1113,6 +1128,7 @@ struct rb_mg {
 namespace rb {
 namespace {
 
+constexpr size_t kMgGraphs = 32;  // recorded shapes a hierarchy keeps
 constexpr int kMgPartials = 4 * K * kMaxGrid;  // 4 quantities x k columns x blocks
 
 template <typename T>
@@ -1535,9 +1551,9 @@ struct Cycle {
   }
 };
 
-// One CG iteration (after the initial z and p): q = A p, x, r update, z = B r, p = z + beta p
+// The first half of a CG iteration: q = A p, x and r updated
 template <typename T, int VEC>
-rb_status cg_iteration(const rb_mg* g, const Cycle<T, VEC>& cy, bool inner, int flexible) {
+rb_status cg_step(const rb_mg* g, const Cycle<T, VEC>& cy, bool inner, cudaGraphConditionalHandle loop) {
   const int k = cy.k, kp = cy.kp;
   const rb_mg_level& l0 = g->lv[0];
   const int64_t n = l0.cells;
@@ -1546,7 +1562,6 @@ rb_status cg_iteration(const rb_mg* g, const Cycle<T, VEC>& cy, bool inner, int 
   T* r = static_cast<T*>(g->r);
   T* p = static_cast<T*>(g->p);
   T* q = static_cast<T*>(g->q);
-  T* z = static_cast<T*>(g->z);
   cudaStream_t s = cy.s;
   if (cy.mf()) {
     auto* kq = &k_mgcg_q<T, VEC, true>;
@@ -1559,22 +1574,38 @@ rb_status cg_iteration(const rb_mg* g, const Cycle<T, VEC>& cy, bool inner, int 
   }
   if (inner) {
     auto* kx = &k_mgcg_xr<T, VEC, true>;
-    kx<<<cy.grid(kx, n), kThreads, 0, s>>>(n, k, kp, x, r, p, q, g->sc, g->partials);
+    kx<<<cy.grid(kx, n), kThreads, 0, s>>>(n, k, kp, x, r, p, q, g->sc, g->partials, loop);
   } else {
     auto* kx = &k_mgcg_xr<T, VEC, false>;
-    kx<<<cy.grid(kx, n), kThreads, 0, s>>>(n, k, kp, x, r, p, q, g->sc, g->partials);
+    kx<<<cy.grid(kx, n), kThreads, 0, s>>>(n, k, kp, x, r, p, q, g->sc, g->partials, loop);
   }
+  RB_CUDA(cudaGetLastError());
+  return RB_OK;
+}
+
+// The second half: z = B r, p = z + beta p
+template <typename T, int VEC>
+rb_status cg_direction(const rb_mg* g, const Cycle<T, VEC>& cy, int flexible) {
+  const int64_t n = g->lv[0].cells;
+  T* z = static_cast<T*>(g->z);
   MgDots dd;
   dd.sc = g->sc;
   dd.partials = g->partials;
-  dd.q = q;
+  dd.q = g->q;
   dd.init = 0;
   dd.flexible = flexible;
-  RB_TRY(cy.run(0, r, z, &dd));
+  RB_TRY(cy.run(0, static_cast<const T*>(g->r), z, &dd));
   auto* kp_ = &k_mgcg_p<T, VEC, false>;
-  kp_<<<cy.grid(kp_, n), kThreads, 0, s>>>(n, k, kp, z, p, g->sc);
+  kp_<<<cy.grid(kp_, n), kThreads, 0, cy.s>>>(n, cy.k, cy.kp, z, static_cast<T*>(g->p), g->sc);
   RB_CUDA(cudaGetLastError());
   return RB_OK;
+}
+
+// One CG iteration (after the initial z and p)
+template <typename T, int VEC>
+rb_status cg_iteration(const rb_mg* g, const Cycle<T, VEC>& cy, bool inner, int flexible) {
+  RB_TRY((cg_step<T, VEC>(g, cy, inner, 0)));
+  return cg_direction<T, VEC>(g, cy, flexible);
 }
 
 // z = B r and p = z (the start of a solve or of a refinement sweep)
@@ -1594,11 +1625,12 @@ rb_status cg_start(const rb_mg* g, const Cycle<T, VEC>& cy) {
 }
 
 struct MgHost {
-  int n_active = 0, n_oactive = 0;
+  int n_active = 0, n_oactive = 0, left = 0;  // as they lie in MgScal
 };
 
 rb_status mg_read(rb_mg* g, MgHost& h, cudaStream_t s) {
-  RB_CUDA(cudaMemcpyAsync(&h.n_active, &g->sc->n_active, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  static_assert(sizeof(MgHost) == 3 * sizeof(int), "read as one piece");
+  RB_CUDA(cudaMemcpyAsync(&h, &g->sc->n_active, sizeof(h), cudaMemcpyDeviceToHost, s));
   RB_CUDA(cudaStreamSynchronize(s));
   return RB_OK;
 }
@@ -1637,6 +1669,87 @@ rb_status run_iterations(rb_mg* g, const Cycle<T, VEC>& cy, bool inner, int flex
   return RB_OK;
 }
 
+// A refinement sweep's scaled FP32 residual, zero d, and the first z and p
+template <int VEC32>
+rb_status sweep_start(const rb_mg* g, const Cycle<float, VEC32>& cy, const rb_cg_params& prm) {
+  const int64_t n = g->lv[0].cells;
+  RB_CUDA(cudaMemsetAsync(g->x, 0, sizeof(float) * (size_t)n * cy.k, cy.s));
+  auto* kr = &k_mg_rhs<float, VEC32, 1>;
+  kr<<<cy.grid(kr, n), kThreads, 0, cy.s>>>(n, cy.k, cy.kp, g->rt, static_cast<float*>(g->r), g->sc, prm.inner_rtol,
+                                           prm.rtol);
+  return cg_start<float, VEC32>(g, cy);
+}
+
+// x += ||r|| d
+template <int VEC32>
+rb_status sweep_end(const rb_mg* g, const Cycle<float, VEC32>& cy) {
+  auto* ka = &k_mg_refine_add<VEC32>;
+  const int64_t n = g->lv[0].cells;
+  ka<<<cy.grid(ka, n), kThreads, 0, cy.s>>>(n, cy.k, cy.kp, g->x64, static_cast<const float*>(g->x), g->sc);
+  RB_CUDA(cudaGetLastError());
+  return RB_OK;
+}
+
+// One refinement sweep's FP32 solve as a graph that ends by itself: the scaled residual, z and p,
+// the first iteration's update, then a loop node whose body is the rest of that iteration and the
+// update of the next, run while columns iterate (k_mgcg_xr decides), and x += ||r|| d.  Replays of a
+// fixed number of iterations with a host check after each ran up to check_every - 1 idle cycles a
+// sweep (about 45 launches of 2 us each) and waited for the host between them. Channel k = 3:
+// 7.70 -> 7.21 ms; projection step on 128^3, m = 2: 22.9 -> 21.0 ms.  exec stays null where the runtime cannot
+// record a loop node (the caller then goes on eagerly).
+template <int VEC32>
+rb_status sweep_graph(rb_mg* g, const Cycle<float, VEC32>& cy, const rb_cg_params& prm, int flexible,
+                      cudaGraphExec_t* exec) {
+  *exec = nullptr;
+  if (!g->cap) RB_CUDA(cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking));
+  Cycle<float, VEC32> cc = cy;
+  cc.s = g->cap;
+  cudaGraph_t graph = nullptr, out = nullptr;
+  RB_CUDA(cudaGraphCreate(&graph, 0));
+  cudaGraphConditionalHandle loop = 0;
+  cudaGraphNodeParams np = {};
+  rb_status st = RB_OK;
+  cudaError_t e = cudaGraphConditionalHandleCreate(&loop, graph, 0, cudaGraphCondAssignDefault);
+  if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(g->cap, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    st = sweep_start<VEC32>(g, cc, prm);
+    if (st == RB_OK) st = cg_step<float, VEC32>(g, cc, true, loop);
+    cudaStreamCaptureStatus cs;
+    cudaGraph_t into = nullptr;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t nd = 0;
+    cudaGraphNode_t node = nullptr;
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = loop;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    if (st == RB_OK) e = cudaStreamGetCaptureInfo(g->cap, &cs, nullptr, &into, &deps, nullptr, &nd);
+    if (st == RB_OK && e == cudaSuccess) e = cudaGraphAddNode(&node, graph, deps, nullptr, nd, &np);
+    if (st == RB_OK && e == cudaSuccess)
+      e = cudaStreamUpdateCaptureDependencies(g->cap, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+    if (st == RB_OK && e == cudaSuccess) st = sweep_end<VEC32>(g, cc);
+    const cudaError_t end = cudaStreamEndCapture(g->cap, &out);
+    if (e == cudaSuccess) e = end;
+  }
+  if (st == RB_OK && e == cudaSuccess) {
+    cudaGraph_t body = np.conditional.phGraph_out[0];
+    e = cudaStreamBeginCaptureToGraph(g->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+      st = cg_direction<float, VEC32>(g, cc, flexible);
+      if (st == RB_OK) st = cg_step<float, VEC32>(g, cc, true, loop);
+      e = cudaStreamEndCapture(g->cap, &out);
+    }
+  }
+  if (st == RB_OK && e == cudaSuccess) e = cudaGraphInstantiate(exec, graph, 0);
+  cudaGraphDestroy(graph);
+  if (st != RB_OK) return st;
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    *exec = nullptr;
+  }
+  return RB_OK;
+}
+
 template <int VEC>
 rb_status true_resid(rb_mg* g, const double* B, int64_t ldb, const double* X, double* out, int kind, int k, int kp,
                      const rb_cg_params& prm, cudaStream_t s) {
@@ -1645,7 +1758,7 @@ rb_status true_resid(rb_mg* g, const double* B, int64_t ldb, const double* X, do
   const int64_t n = g->lv[0].cells;
   const int grid = wave_grid(kern, (n + kThreads / kp - 1) / (kThreads / kp));
   kern<<<grid, kThreads, 0, s>>>(csr_args<double>(A, X, nullptr, k, kp), B, ldb, out, kind, prm.project_mean,
-                                 prm.rtol * prm.rtol, g->sc, g->partials);
+                                 prm.rtol * prm.rtol, prm.max_iter, g->sc, g->partials);
   RB_CUDA(cudaGetLastError());
   return RB_OK;
 }
@@ -1694,35 +1807,49 @@ rb_status mg_solve_vec(rb_mg* g, const rb_cg_params& prm, const double* B, int64
     Cycle<float, VEC32> cy{g, k, kp32, s, &g->sc->n_active};
     double* x64 = g->x64;
     k_mg_copy<double, double><<<cg, 256, 0, s>>>(n, k, X, ldx, x64, k);
-    int total_inner = 0;
+    // the sweep's graph, kept per shape and inner tolerance; the hierarchy's first sweep of a shape
+    // runs eagerly, so that the launch-shape caches are filled before the recording
+    uint64_t tol_bits;
+    std::memcpy(&tol_bits, &prm.inner_rtol, 8);
+    const std::vector<int> key = {-1, k, flexible, (int)(uint32_t)tol_bits, (int)(uint32_t)(tol_bits >> 32)};
     for (;; ++sweeps) {
       RB_TRY(true_resid<VEC64>(g, B, ldb, x64, g->rt, sweeps == 0 ? TR_INIT : TR_CHECK, k, kp64, prm, s));
       ++spmm64;
       RB_TRY(mg_read(g, h, s));
       ++syncs;
       if (h.n_oactive == 0) break;
-      if (sweeps >= prm.max_sweeps || total_inner >= prm.max_iter) {
+      if (sweeps >= prm.max_sweeps || h.left <= 0) {
         k_mg_mark_noconv<<<1, K, 0, s>>>(g->sc, k);
         break;
       }
-      RB_CUDA(cudaMemsetAsync(g->x, 0, sizeof(float) * (size_t)n * k, s));
-      auto* kr = &k_mg_rhs<float, VEC32, 1>;
-      kr<<<cy.grid(kr, n), kThreads, 0, s>>>(n, k, kp32, g->rt, static_cast<float*>(g->r), g->sc, prm.inner_rtol,
-                                            prm.rtol);
-      RB_TRY((cg_start<float, VEC32>(g, cy)));
-      int it = 0;
+      auto it = g->graphs.find(key);
+      if (it != g->graphs.end() && !it->second) {
+        if (g->graphs.size() > kMgGraphs)  // other shapes and tolerances: recorded again when they return
+          for (auto o = g->graphs.begin(); o != g->graphs.end();) {
+            if (o == it || !o->second) {
+              ++o;
+            } else {
+              RB_CUDA(cudaStreamSynchronize(s));
+              cudaGraphExecDestroy(o->second);
+              o = g->graphs.erase(o);
+            }
+          }
+        RB_TRY(sweep_graph<VEC32>(g, cy, prm, flexible, &it->second));
+      }
+      if (it != g->graphs.end() && it->second) {
+        RB_CUDA(cudaGraphLaunch(it->second, s));
+        continue;
+      }
+      g->graphs.emplace(key, nullptr);
+      RB_TRY(sweep_start<VEC32>(g, cy, prm));
       for (;;) {
         RB_TRY(mg_read(g, h, s));
         ++syncs;
-        if (h.n_active == 0 || total_inner + it >= prm.max_iter) break;
-        const int chunk = std::min(check, prm.max_iter - total_inner - it);
-        RB_TRY((run_iterations<float, VEC32>(g, cy, true, flexible, chunk, uses)));
-        it += chunk;
+        if (h.n_active == 0 || h.left <= 0) break;
+        const int chunk = std::min(check, h.left);
+        for (int i = 0; i < chunk; ++i) RB_TRY((cg_iteration<float, VEC32>(g, cy, true, flexible)));
       }
-      total_inner += it;
-      auto* ka = &k_mg_refine_add<VEC32>;
-      ka<<<cy.grid(ka, n), kThreads, 0, s>>>(n, k, kp32, x64, static_cast<const float*>(g->x), g->sc);
-      RB_CUDA(cudaGetLastError());
+      RB_TRY(sweep_end<VEC32>(g, cy));
     }
     if (prm.project_mean) {
       auto* kc = &k_mg_colsum<VEC64>;
