@@ -60,6 +60,108 @@ __global__ void __launch_bounds__(kThreads) k_spmm_stencil7_run(Stencil7<T> st, 
   }
 }
 
+// The FP64 product.  It is bound by the FP64 pipe (2 multiply-adds per clock and SM), so what counts
+// is FP64 operations per value.  The factors fixed on an x line (fixed y, z) and on an x cell are
+// tabulated when the operator is made, with its scale:
+//   line: a = s w_y w_z, b_ym, b_yp = s w_z / d_y, b_zm, b_zp = s w_y / d_z, S = -(b_ym + ... + b_zp)
+//   cell: 1 / d_x below and above, their negated sum D, w_x
+// One or two columns per thread: y = a (x_- / d + x_+ / d + D x_0) + w_x (b . x_yz + S x_0), ten
+// operations a value and none per cell.  More columns: the seven entries formed first (8 operations
+// a cell: two products with a, four with w_x, and the diagonal's two), then seven a value.  Forming
+// entries and diagonal from the axis tables took 14 a cell and 8 a value.  190 x 127 x 95 (one cell
+// per thread before), k = 3: 162 -> 121 us (the pipe alone: 106); 192 x 128 x 96 (runs of four cells
+// before), k = 1, 2, 3, 4, 8: 97, 131, 169, 250, 490 -> 45, 86, 123, 168, 332 us.
+struct alignas(16) LineCoef {
+  double a, bym, byp, bzm, bzp, s;
+};
+struct alignas(16) CellCoef {
+  double m, p, d, w;
+};
+
+template <int VEC, bool SCALE>
+__global__ void __launch_bounds__(kThreads) k_spmm_stencil7_f64(Stencil7<double> st, const LineCoef* __restrict__ lines,
+                                                                 const CellCoef* __restrict__ cells, int64_t n, int k,
+                                                                 int kp, const double* __restrict__ X, int64_t ldx,
+                                                                 double* __restrict__ Y, int64_t ldy,
+                                                                 const double* __restrict__ cs) {
+  const int R = kThreads / kp;
+  const int chunk = threadIdx.x % kp;
+  if (chunk * VEC >= k) return;
+  double c[VEC];
+#pragma unroll
+  for (int q = 0; q < VEC; ++q) c[q] = SCALE ? cs[chunk * VEC + q] : 1.0;
+  const int nx = st.n[0], ny = st.n[1], nz = st.n[2], plane = nx * ny;
+  const double* xc = X + chunk * VEC;
+  for (int64_t row = (int64_t)blockIdx.x * R + threadIdx.x / kp; row < n; row += (int64_t)gridDim.x * R) {
+    const uint32_t r32 = (uint32_t)row;
+    const int line = (int)st.dx.div(r32), i = (int)(r32 - (uint32_t)line * (uint32_t)nx);
+    const int z = (int)st.dxy.div(r32), j = line - z * ny;
+    // neighbour rows (at a wall the factor is 0 and the own row is read)
+    const int om = i > 0 ? -1 : (st.per[0] ? nx - 1 : 0), op = i + 1 < nx ? 1 : (st.per[0] ? 1 - nx : 0);
+    const int jm = j > 0 ? -nx : (st.per[1] ? plane - nx : 0), jp = j + 1 < ny ? nx : (st.per[1] ? nx - plane : 0);
+    const int zm = z > 0 ? -plane : (st.per[2] ? (nz - 1) * plane : 0);
+    const int zp = z + 1 < nz ? plane : (st.per[2] ? -(nz - 1) * plane : 0);
+    const Vec<double, VEC> x0 = ldv<double, VEC>(xc + row * ldx);
+    const Vec<double, VEC> xm = ldv<double, VEC>(xc + (row + om) * ldx), xp = ldv<double, VEC>(xc + (row + op) * ldx);
+    const Vec<double, VEC> ym = ldv<double, VEC>(xc + (row + jm) * ldx), yp = ldv<double, VEC>(xc + (row + jp) * ldx);
+    const Vec<double, VEC> um = ldv<double, VEC>(xc + (row + zm) * ldx), up = ldv<double, VEC>(xc + (row + zp) * ldx);
+    const CellCoef t = cells[i];
+    const LineCoef l = lines[line];
+    Vec<double, VEC> y;
+    if constexpr (VEC <= 2) {
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) {
+        const double u = fma(t.d, x0.v[q], fma(t.p, xp.v[q], t.m * xm.v[q]));
+        double v = l.s * x0.v[q];
+        v = fma(l.bym, ym.v[q], v);
+        v = fma(l.byp, yp.v[q], v);
+        v = fma(l.bzm, um.v[q], v);
+        v = fma(l.bzp, up.v[q], v);
+        y.v[q] = fma(l.a, u, t.w * v);
+      }
+    } else {
+      const double cxm = l.a * t.m, cxp = l.a * t.p, cym = t.w * l.bym, cyp = t.w * l.byp, czm = t.w * l.bzm,
+                   czp = t.w * l.bzp, diag = fma(t.w, l.s, l.a * t.d);
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) {
+        double v = diag * x0.v[q];
+        v = fma(cxm, xm.v[q], v);
+        v = fma(cxp, xp.v[q], v);
+        v = fma(cym, ym.v[q], v);
+        v = fma(cyp, yp.v[q], v);
+        v = fma(czm, um.v[q], v);
+        y.v[q] = fma(czp, up.v[q], v);
+      }
+    }
+    if constexpr (SCALE) {
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) y.v[q] *= c[q];
+    }
+    stv<double, VEC>(Y + row * ldy + chunk * VEC, y);
+  }
+}
+
+// the tables of k_spmm_stencil7_f64: lines (y fastest), then x cells
+__global__ void k_stencil7_lines(Stencil7<double> st, LineCoef* __restrict__ lines, CellCoef* __restrict__ cells) {
+  const int ny = st.n[1], n_lines = ny * st.n[2];
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n_lines + st.n[0]; t += gridDim.x * blockDim.x) {
+    if (t < n_lines) {
+      const int z = t / ny, j = t - z * ny;
+      const double wy = st.scale * st.w[1][j], wz = st.scale * st.w[2][z];
+      LineCoef l;
+      l.a = wy * st.w[2][z];
+      l.bym = wz * st.ic[1][j], l.byp = wz * st.ic[1][j + 1];
+      l.bzm = wy * st.ic[2][z], l.bzp = wy * st.ic[2][z + 1];
+      l.s = -((l.bym + l.byp) + (l.bzm + l.bzp));
+      lines[t] = l;
+    } else {
+      const int i = t - n_lines;
+      const double m = st.ic[0][i], p = st.ic[0][i + 1];
+      cells[i] = CellCoef{m, p, -(m + p), st.w[0][i]};
+    }
+  }
+}
+
 // Jacobi diagonal of the operator in both precisions (as rb_operator_create forms it from the
 // FP64 diagonal): 1 / a_ii and the FP32 reciprocal of the FP32-rounded entry
 __global__ void k_stencil7_dinv(Stencil7<double> st, int64_t n, double* __restrict__ d64, float* __restrict__ d32) {
@@ -84,8 +186,25 @@ Stencil7<T> view(const rb_op* op) {
   return s;
 }
 
-template <typename T, int VEC>
-rb_status launch(const rb_op* op, const SpmmSched& sc, const T* X, int64_t ldx, T* Y, int64_t ldy, int k,
+template <int VEC>
+rb_status launch(const rb_op* op, const SpmmSched& sc, const double* X, int64_t ldx, double* Y, int64_t ldy, int k,
+                 const double* cs, cudaStream_t s) {
+  const int R = kThreads / sc.kp;
+  const int64_t blocks = ((int64_t)op->n_rows + R - 1) / R;
+  const LineCoef* lines = reinterpret_cast<const LineCoef*>(op->st_lines);
+  const CellCoef* cells = reinterpret_cast<const CellCoef*>(lines + (size_t)op->st_n[1] * op->st_n[2]);
+  auto go = [&](auto* kern) {
+    kern<<<wave_grid(kern, blocks), kThreads, 0, s>>>(view<double>(op), lines, cells, op->n_rows, k, sc.kp, X, ldx, Y, ldy,
+                                                      cs);
+  };
+  if (cs) go(&k_spmm_stencil7_f64<VEC, true>);
+  else go(&k_spmm_stencil7_f64<VEC, false>);
+  RB_CUDA(cudaGetLastError());
+  return RB_OK;
+}
+
+template <int VEC>
+rb_status launch(const rb_op* op, const SpmmSched& sc, const float* X, int64_t ldx, float* Y, int64_t ldy, int k,
                  const double* cs, cudaStream_t s) {
   const int R = kThreads / sc.kp;
   constexpr int RUN = 4;
@@ -97,25 +216,25 @@ rb_status launch(const rb_op* op, const SpmmSched& sc, const T* X, int64_t ldx, 
     drow.init((uint32_t)op->st_n[1]);
     const bool contig = sc.kp == 1 && ldx == VEC && ldy == VEC && ((uintptr_t)X % 16) == 0 && ((uintptr_t)Y % 16) == 0;
     auto go = [&](auto kern) {
-      kern<<<wave_grid(kern, rblocks), kThreads, 0, s>>>(view<T>(op), drun, drow, n_runs, k, sc.kp, X, ldx, Y, ldy, cs);
+      kern<<<wave_grid(kern, rblocks), kThreads, 0, s>>>(view<float>(op), drun, drow, n_runs, k, sc.kp, X, ldx, Y, ldy, cs);
     };
     if (cs) {
-      if (contig) go(&k_spmm_stencil7_run<T, VEC, RUN, true, true>);
-      else go(&k_spmm_stencil7_run<T, VEC, RUN, true, false>);
+      if (contig) go(&k_spmm_stencil7_run<float, VEC, RUN, true, true>);
+      else go(&k_spmm_stencil7_run<float, VEC, RUN, true, false>);
     } else {
-      if (contig) go(&k_spmm_stencil7_run<T, VEC, RUN, false, true>);
-      else go(&k_spmm_stencil7_run<T, VEC, RUN, false, false>);
+      if (contig) go(&k_spmm_stencil7_run<float, VEC, RUN, false, true>);
+      else go(&k_spmm_stencil7_run<float, VEC, RUN, false, false>);
     }
     RB_CUDA(cudaGetLastError());
     return RB_OK;
   }
   const int64_t blocks = ((int64_t)op->n_rows + R - 1) / R;
   if (cs) {
-    auto* kern = &k_spmm_stencil7<T, VEC, true>;
-    kern<<<wave_grid(kern, blocks), kThreads, 0, s>>>(view<T>(op), op->n_rows, k, sc.kp, X, ldx, Y, ldy, cs);
+    auto* kern = &k_spmm_stencil7<float, VEC, true>;
+    kern<<<wave_grid(kern, blocks), kThreads, 0, s>>>(view<float>(op), op->n_rows, k, sc.kp, X, ldx, Y, ldy, cs);
   } else {
-    auto* kern = &k_spmm_stencil7<T, VEC, false>;
-    kern<<<wave_grid(kern, blocks), kThreads, 0, s>>>(view<T>(op), op->n_rows, k, sc.kp, X, ldx, Y, ldy, cs);
+    auto* kern = &k_spmm_stencil7<float, VEC, false>;
+    kern<<<wave_grid(kern, blocks), kThreads, 0, s>>>(view<float>(op), op->n_rows, k, sc.kp, X, ldx, Y, ldy, cs);
   }
   RB_CUDA(cudaGetLastError());
   return RB_OK;
@@ -127,10 +246,10 @@ rb_status launch_t(const rb_op* op, const SpmmSched& sc, const void* X, int64_t 
   const T* x = static_cast<const T*>(X);
   T* y = static_cast<T*>(Y);
   switch (sc.vec) {
-    case 1: return launch<T, 1>(op, sc, x, ldx, y, ldy, k, cs, s);
-    case 2: return launch<T, 2>(op, sc, x, ldx, y, ldy, k, cs, s);
-    case 3: return launch<T, 3>(op, sc, x, ldx, y, ldy, k, cs, s);
-    case 4: return launch<T, 4>(op, sc, x, ldx, y, ldy, k, cs, s);
+    case 1: return launch<1>(op, sc, x, ldx, y, ldy, k, cs, s);
+    case 2: return launch<2>(op, sc, x, ldx, y, ldy, k, cs, s);
+    case 3: return launch<3>(op, sc, x, ldx, y, ldy, k, cs, s);
+    case 4: return launch<4>(op, sc, x, ldx, y, ldy, k, cs, s);
   }
   set_error("spmm: unsupported vector width %d", sc.vec);
   return RB_EUNSUPPORTED;
@@ -195,6 +314,9 @@ extern "C" rb_status rb_fvm_stencil_create(const rb_grid_desc* grid, double scal
     alloc((void**)&w32[d], n * 4);
     alloc((void**)&ic32[d], n * 4);
   }
+  if (dtype == RB_F64)
+    alloc((void**)&op->st_lines,
+          sizeof(LineCoef) * (size_t)grid->n[1] * grid->n[2] + sizeof(CellCoef) * (size_t)grid->n[0]);
   alloc((void**)&op->err, sizeof(int));
   alloc((void**)&op->dinv64, (size_t)nr * 8);
   alloc((void**)&op->dinv32, (size_t)nr * 4);
@@ -206,6 +328,12 @@ extern "C" rb_status rb_fvm_stencil_create(const rb_grid_desc* grid, double scal
     v.init_div();
     const int grid_blocks = (int)std::min<int64_t>(((int64_t)nr + 255) / 256, kMaxGrid);
     k_stencil7_dinv<<<grid_blocks, 256, 0, s>>>(v, nr, op->dinv64, op->dinv32);
+    if (op->st_lines) {
+      LineCoef* lines = reinterpret_cast<LineCoef*>(op->st_lines);
+      const int64_t entries = (int64_t)grid->n[1] * grid->n[2] + grid->n[0];
+      k_stencil7_lines<<<(int)std::min<int64_t>((entries + 127) / 128, kMaxGrid), 128, 0, s>>>(
+          v, lines, reinterpret_cast<CellCoef*>(lines + (size_t)grid->n[1] * grid->n[2]));
+    }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) st = cuda_fail(e, "stencil operator tables", __FILE__, __LINE__);
