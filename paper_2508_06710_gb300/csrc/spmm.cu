@@ -55,28 +55,69 @@ std::vector<int> vec_candidates(int eb, int k) {
 
 }  // namespace
 
+// The schedule of a call that nobody tuned.  Width: 16-byte vectors with one thread per row, then
+// three columns, then the widest aligned vector.  The other choices by measurement (us; channel
+// 192 x 128 x 96 Laplacian L, gradient G and divergence, 160^3 13- and 27-point operators, the
+// extruded mesh):
+//   long rows (12 to 40 entries: the 13- and 27-point operators').  FP32: the TMA ring, whose entries
+//     come from shared memory while eight or more gathers per lane are in flight (27p k = 1, 3, 8
+//     137, 163, 211 and with the row split over lanes 185, 224, 353; 13p k = 1, 3 74, 86 and 91, 107;
+//     not 13p k = 8, 140 and direct 134; 27p k = 4 in halves, 164 against 168).  FP64 is
+//     bound by its pipe and splitting a row pays shuffles on it: one lane per row, in the ring where
+//     loads still matter (27p k = 1, 2, 3 239, 380, 570 and direct 291, 397, 662; 13p k = 1 109 and
+//     129), direct otherwise (13p k = 3 275, in the ring 292; with eight lanes per row, the choice
+//     before, 1129).  Longer rows than these operators', and few rows (24^3: too few for one lane each
+//     to hide its gathers, 27p FP32 k = 3 3.4 and in the ring 5.2), keep up to eight lanes.
+//   grid, direct kernels.  FP64 with two columns or more: one block per row block, not a resident
+//     wave (L k = 3 91 and 97, k = 8 226 and 248, extruded k = 64 150 and 157); one column and the
+//     gradient's rows of two: the wave (G k = 3 86 and 93).  FP32: the wave.
+//   width.  FP64 k = 4, 8, 16, 32 on short rows: four doubles a thread (G k = 4 107 and 115, the
+//     divergence k = 8 191 and 224 with the grid).
+//   the TMA ring on short rows.  FP32, a matrix that does not stay in L2, and little work per entry
+//     loaded (rows of two: G k = 3 49 and 58) or many columns (L k = 16 88 and 99).
+// The ring is taken only where every tile fits its stages (no row far above the average).
 SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X, const void* Y) {
   const int eb = op->dtype == RB_F32 ? 4 : 8;
+  const bool f64 = op->dtype == RB_F64, f32 = op->dtype == RB_F32;
+  const bool csr = op->format == RB_CSR && op->ext_nz == 0;
+  const double len = op->avg_row_len;
+  const bool even = op->max_row_len <= 1.25 * len + 1.0;  // every tile within the ring's capacity
+  const bool mid = csr && len >= 12.0 && len < 40.0 && (f64 || f32) && op->n_rows > 24000;
+  const bool many = csr && f32 && k >= 12 && k % 4 == 0 && len < 12.0;
   SpmmSched sc;
   sc.lpr = 1;
   sc.stage = 0;
   sc.grid_cap = -1;
-  // preference: 16-byte vectors with one thread per row, then 3-wide, then the widest aligned vector
   std::vector<int> order;
+  if (mid && len >= 20.0 && (f64 ? k == 2 : k == 4)) order.push_back(k / 2);
+  // (up to 32 columns: beyond, unaligned rows are refused, and four doubles need no alignment)
+  if (csr && f64 && k % 4 == 0 && (k & (k - 1)) == 0 && k <= 32 && len < 12.0) order.push_back(4);
+  if (many) order.push_back(4);
   if (k * eb == 16 || k * eb == 8) order.push_back(k);
   if (k % 3 == 0 && k <= 12) order.push_back(3);
   for (int w = 16 / eb; w >= 1; w >>= 1) order.push_back(w);
-  if (eb == 8 && k == 4) order.insert(order.begin(), 2);
+  if (eb == 8 && k == 4 && order[0] != 4) order.insert(order.begin(), 2);
   for (int w : order) {
     SpmmSched t = sc;
     t.vec = w;
     if (k % w) continue;
     t.kp = next_pow2(k / w);
-    if (sched_valid(op, t, k, ldx, ldy, X, Y)) {
-      if (op->format != RB_SELL && op->avg_row_len >= 12.0) t.lpr = std::max(1, std::min(8, 32 / t.kp / 4));
+    if (!sched_valid(op, t, k, ldx, ldy, X, Y)) continue;
+    if (!mid && op->format != RB_SELL && len >= 12.0) {
+      t.lpr = std::max(1, std::min(8, 32 / t.kp / 4));
       if (!sched_valid(op, t, k, ldx, ldy, X, Y)) t.lpr = 1;
-      return t;
     }
+    if (op->format == RB_CSR && f64 && k >= 2 && len >= 4.0) t.grid_cap = 0;
+    const double matrix = (double)op->nnz * (4 + eb) + 4.0 * op->n_rows;
+    const bool ring = mid ? (f32 ? k < 8 || len >= 20.0 : k == 1 || (len >= 20.0 && k <= 3))
+                          : csr && f32 && matrix > 100e6 && (len < 4.0 || (many && w == 4)) && op->n_rblk <= 1;
+    if (ring && even) {
+      SpmmSched r = t;
+      r.stage = 2;
+      r.grid_cap = 0;
+      if (sched_valid(op, r, k, ldx, ldy, X, Y)) t = r;
+    }
+    return t;
   }
   sc.vec = 1;
   sc.kp = next_pow2(k);

@@ -85,15 +85,21 @@ rb_status launch_csr(const rb_op* op, const SpmmSched& sc, const T* X, int64_t l
   if (grid == 0) return RB_OK;
   if (sc.stage == 2) {
     if constexpr (LPR == 1) {
-      auto* kern = &k_spmm_tma<T, VEC, EPI>;
-      const int cap = tma_capacity<T>(op, R, kTmaSmemLimit);
-      const size_t smem = tma_layout<T>(R, cap).total;
-      RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem));
-      grid = wave_grid(kern, grid, smem, kTmaThreads);
-      if (sc.grid_cap > 0) grid = std::min<int64_t>(grid, sc.grid_cap);  // fewer blocks, more tiles each
-      kern<<<(unsigned)grid, kTmaThreads, smem, s>>>(a, R, cap, op->err);
-      RB_CUDA(cudaGetLastError());
-      return RB_OK;
+      auto go = [&](auto* kern, int rows, int cap, size_t smem, int threads) -> rb_status {
+        RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem));
+        grid = wave_grid(kern, ((int64_t)op->n_rows + rows - 1) / rows, smem, threads);
+        if (sc.grid_cap > 0) grid = std::min<int64_t>(grid, sc.grid_cap);  // fewer blocks, more tiles each
+        kern<<<(unsigned)grid, threads, smem, s>>>(a, rows, cap, op->err);
+        RB_CUDA(cudaGetLastError());
+        return RB_OK;
+      };
+      if (op->avg_row_len >= 12.0) {
+        const int consumers = tma_long_threads(op->avg_row_len, sizeof(T), sc.kp), rows = consumers / sc.kp;
+        const int cap = tma_capacity<T, true>(op, rows, kTmaSmemLimit);
+        return go(&k_spmm_tma<T, VEC, EPI, true>, rows, cap, tma_layout<T, true>(rows, cap).total, consumers + 32);
+      }
+      const int cap = tma_capacity<T, false>(op, R, kTmaSmemLimit);
+      return go(&k_spmm_tma<T, VEC, EPI, false>, R, cap, tma_layout<T, false>(R, cap).total, kTmaThreads);
     }
     set_error("spmm: the TMA pipeline takes one lane per row");
     return RB_EUNSUPPORTED;

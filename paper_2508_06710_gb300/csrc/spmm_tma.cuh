@@ -20,8 +20,25 @@
 
 namespace rb {
 
-constexpr int kTmaStages = 3;
+// Two shapes of the ring.  Short rows: three stages and a block's usual 256 consumer threads.  Long
+// rows (LONG): a tile is tens of KB, so two stages and as many consumers as keep a tile near 28 KB
+// (four blocks per SM), and each lane issues kLongGathers gathers before it uses the first: a row's
+// gathers are an L2 round trip each, and two at a time left the 16 resident consumer warps waiting.
+// 160^3 27-point operator, FP32 k = 8: 211 us (1.16 GB: 0.82 of the measured HBM rate; three blocks
+// per SM, left to itself the compiler fits two: 254); with three stages 347, two gathers at a time
+// over 380, direct with eight threads a row 353; 13-point, k = 4: 90 us against 105 (direct).
+template <bool LONG>
+constexpr int kTmaStages = LONG ? 2 : 3;
+template <typename T, int VEC>
+constexpr int kLongGathers = sizeof(T) * VEC >= 12 ? 8 : 13;
 constexpr int kTmaThreads = kThreads + 32;  // 8 consumer warps + 1 producer warp
+
+// consumer threads of a long-row block: 256, halved while its tile exceeds 32 KB
+inline int tma_long_threads(double avg_row_len, int elem_bytes, int kp) {
+  int c = kThreads;
+  while (c > 64 && c / 2 >= kp && (double)(c / kp) * avg_row_len * (4 + elem_bytes) > 32 * 1024) c /= 2;
+  return c;
+}
 
 __host__ __device__ inline size_t align128(size_t v) { return (v + 127) & ~(size_t)127; }
 
@@ -30,7 +47,7 @@ struct TmaLayout {
   size_t rp_off, ci_off, va_off, stage_bytes, hdr_off, bar_off, total;
 };
 
-template <typename T>
+template <typename T, bool LONG>
 __host__ __device__ inline TmaLayout tma_layout(int R, int cap) {
   TmaLayout L;
   L.R = R;
@@ -43,41 +60,44 @@ __host__ __device__ inline TmaLayout tma_layout(int R, int cap) {
   L.va_off = off;
   off += align128((size_t)cap * sizeof(T));
   L.stage_bytes = off;
-  L.hdr_off = kTmaStages * L.stage_bytes;
+  L.hdr_off = kTmaStages<LONG> * L.stage_bytes;
   L.bar_off = L.hdr_off + 128;
-  L.total = L.bar_off + 2 * kTmaStages * sizeof(uint64_t);
+  L.total = L.bar_off + 2 * kTmaStages<LONG> * sizeof(uint64_t);
   return L;
 }
 
 // Staged nonzeros per stage: 1.25x the average row plus slack, a multiple of 4, and the
 // whole ring within `limit` bytes of shared memory.
-template <typename T>
+template <typename T, bool LONG>
 inline int tma_capacity(const rb_op* op, int R, size_t limit) {
   int cap = round4((int)((double)R * (op->avg_row_len * 1.25 + 1.0)) + 16);
-  while (cap > 16 && tma_layout<T>(R, cap).total > limit) cap -= 16;
+  if (LONG && (double)R * op->max_row_len < cap - 16) cap = round4(R * op->max_row_len) + 16;
+  while (cap > 16 && tma_layout<T, LONG>(R, cap).total > limit) cap -= 16;
   return cap;
 }
 
-template <typename T, int VEC, int EPI>
-__global__ void __launch_bounds__(kTmaThreads) k_spmm_tma(CsrArgs<T> a, int R, int cap, int* __restrict__ err) {
+template <typename T, int VEC, int EPI, bool LONG>
+__global__ void __launch_bounds__(kTmaThreads, LONG ? (sizeof(T) == 4 ? 3 : 2) : 0) k_spmm_tma(CsrArgs<T> a, int R, int cap, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char sm[];
-  const TmaLayout L = tma_layout<T>(R, cap);
+  constexpr int kStages = kTmaStages<LONG>;
+  const int consumers = (int)blockDim.x - 32;
+  const TmaLayout L = tma_layout<T, LONG>(R, cap);
   int* hdr = reinterpret_cast<int*>(sm + L.hdr_off);  // per stage: first staged nonzero, staged flag
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + L.bar_off);
-  uint64_t* empty = full + kTmaStages;
+  uint64_t* empty = full + kStages;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_tiles = (a.n_rows + R - 1) / R;
   const int my_tiles = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kTmaStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], kThreads / 32);
+      mbar_init(&empty[s], consumers / 32);
     }
     fence_barrier_init();
   }
   __syncthreads();
 
-  if (warp == kThreads / 32) {
+  if (warp == consumers / 32) {
     // ------------------------------------------------------------------- producer warp
     int b = 0, e = 0;
     int armed = 0;
@@ -93,8 +113,8 @@ __global__ void __launch_bounds__(kTmaThreads) k_spmm_tma(CsrArgs<T> a, int R, i
       const int p0 = __shfl_sync(0xffffffffu, b, i & 31);
       const int p1 = __shfl_sync(0xffffffffu, e, i & 31);
       if (lane == 0) {
-        const int s = i % kTmaStages;
-        const uint32_t ph = (uint32_t)(i / kTmaStages) & 1u;
+        const int s = i % kStages;
+        const uint32_t ph = (uint32_t)(i / kStages) & 1u;
         if (!mbar_wait(&empty[s], ph ^ 1u)) {
           atomicExch(err, 1);
           ok = 0;
@@ -124,8 +144,8 @@ __global__ void __launch_bounds__(kTmaThreads) k_spmm_tma(CsrArgs<T> a, int R, i
     }
     // no copy may be in flight when the block exits
     if (lane == 0) {
-      for (int i = armed > kTmaStages ? armed - kTmaStages : 0; i < armed; ++i)
-        if (!mbar_wait(&full[i % kTmaStages], (uint32_t)(i / kTmaStages) & 1u)) atomicExch(err, 2);
+      for (int i = armed > kStages ? armed - kStages : 0; i < armed; ++i)
+        if (!mbar_wait(&full[i % kStages], (uint32_t)(i / kStages) & 1u)) atomicExch(err, 2);
     }
     return;
   }
@@ -134,8 +154,8 @@ __global__ void __launch_bounds__(kTmaThreads) k_spmm_tma(CsrArgs<T> a, int R, i
   const int chunk = threadIdx.x % a.kp;
   const int rloc = threadIdx.x / a.kp;
   for (int i = 0; i < my_tiles; ++i) {
-    const int s = i % kTmaStages;
-    const uint32_t ph = (uint32_t)(i / kTmaStages) & 1u;
+    const int s = i % kStages;
+    const uint32_t ph = (uint32_t)(i / kStages) & 1u;
     const bool got = mbar_wait(&full[s], ph);
     if (!__all_sync(0xffffffffu, got)) {  // leave as a whole warp
       if (lane == 0) atomicExch(err, 3);
@@ -158,8 +178,33 @@ __global__ void __launch_bounds__(kTmaThreads) k_spmm_tma(CsrArgs<T> a, int R, i
       const int re = s_rp[rloc + 1] - p0a;
       const T* Xc = a.X + chunk * VEC;
       if (staged) {
+        int p = rs;
+        if constexpr (LONG) {
+          // FP32: two running sums, for a smaller rounding error than one; FP64: one (a further
+          // addition would take a slot of its pipe)
+          constexpr int U = kLongGathers<T, VEC>, A = sizeof(T) == 4 ? 2 : 1;
+          T part[A][VEC];
+#pragma unroll
+          for (int q = 0; q < A; ++q)
+#pragma unroll
+            for (int ee = 0; ee < VEC; ++ee) part[q][ee] = T(0);
+          for (; p + U <= re; p += U) {
+            Vec<T, VEC> x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) x[u] = ldv<T, VEC>(Xc + (int64_t)s_ci[p + u] * a.ldx);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const T v = s_va[p + u];
+#pragma unroll
+              for (int ee = 0; ee < VEC; ++ee) part[u % A][ee] = fma(v, x[u].v[ee], part[u % A][ee]);
+            }
+          }
+#pragma unroll
+          for (int ee = 0; ee < VEC; ++ee)
+            acc[ee] = A == 2 ? part[0][ee] + part[1 % A][ee] : part[0][ee];
+        }
 #pragma unroll 2
-        for (int p = rs; p < re; ++p) {
+        for (; p < re; ++p) {
           const int c = s_ci[p];
           const T v = s_va[p];
           const Vec<T, VEC> x = ldv<T, VEC>(Xc + (int64_t)c * a.ldx);
