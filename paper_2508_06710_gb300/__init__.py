@@ -220,20 +220,30 @@ def fma_peak(dtype="f64", stream=None) -> float:
 
 
 # ----------------------------------------------------------------------------- tensor helpers
-def _torch():
-    import torch
+_torch_module = None
 
-    return torch
+
+def _torch():
+    global _torch_module
+    if _torch_module is None:
+        import torch
+
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream(stream=None):
+    """The stream's handle as an integer (what a c_void_p argument takes).  The current stream's is
+    asked for directly: the Stream object that torch.cuda.current_stream() builds costs more host
+    time (5 us) than the library's whole call."""
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _block(t, name, pairs=False):
@@ -246,15 +256,20 @@ def _block(t, name, pairs=False):
         if not t.is_cuda:
             raise ValueError(f"{name} must be a CUDA tensor")
         return t, t.shape[0], t.shape[1], max(t.stride(0) // 2, t.shape[1])
-    if t.dim() == 3:
+    shape = t.shape
+    if len(shape) == 3:
         raise ValueError(f"{name}: a double-float block goes only to a df64 operator or df_join")
-    if t.dim() == 1:
+    if len(shape) == 1:
         t = t.view(-1, 1)
-    if t.dim() != 2 or t.stride(1) != 1:
+        shape = t.shape
+    strides = t.stride()
+    if len(shape) != 2 or strides[1] != 1:
         raise ValueError(f"{name} must be a 2-D tensor with contiguous rows (stride (ld, 1))")
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
-    return t, t.shape[0], t.shape[1], max(t.stride(0), t.shape[1])
+    n, k = shape
+    ld = strides[0]
+    return t, n, k, (ld if ld > k else k)
 
 
 def _dtype_code(t):
@@ -435,7 +450,9 @@ class Operator:
             shape = (self.n_rows, X.shape[1], 2) if self.dtype == "df64" else (self.n_rows, X.shape[1] if X.dim() > 1 else 1)
             Y = torch.empty(shape, dtype=X.dtype, device=X.device)
         X, k, ldx, Y, ldy = self._blocks(X, Y)
-        _check(lib().rb_spmm(self.handle, _ptr(X), ldx, _ptr(Y), ldy, k, _ptr(c), _stream(stream)), "rb_spmm")
+        st = lib().rb_spmm(self.handle, X.data_ptr(), ldx, Y.data_ptr(), ldy, k, _ptr(c), _stream(stream))
+        if st:
+            _check(st, "rb_spmm")
         return Y
 
     def tune(self, X, Y, stream=None):
