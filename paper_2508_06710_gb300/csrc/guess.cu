@@ -517,6 +517,233 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_row(Conv3Args a, int chu
   if (warp == 0) tmem_dealloc(tmem, kCols);
 }
 
+// ------------------------------- 3x3x3 convolution on 128-cell rows, marching planes (MMA)
+//
+// The row kernel above issues 18 (8 input channels) or 27 (16) MMAs of N = 16 per output row, and
+// an MMA costs 32 + N / 4 cycles.  Here N holds every output row that an input line contributes to,
+// up to nine: a CTA owns kPlaneRows rows y and marches z; A is line (zz, y) and B stacks, for each
+// of the CTA's rows y - 1 .. y + 1, the weights towards planes zz - 1, zz and zz + 1 as column blocks
+// that add to those planes' accumulators.  2 (or 3) MMAs per input line of N <= 96 (144) and 1.5
+// lines per output row: 144 cycles per output row and plane where 18 MMAs take 650, and 1.5 lines
+// loaded instead of 3.3.
+//
+// Accumulators: a row has three column blocks of CB = 8 or 16 channels, plane z in block z mod 3 (CB =
+// 8: and a fourth, unused, under zero weights: N must be a multiple of 16).  Which plane a block
+// belongs to turns with zz, so B is kept three times, one per zz mod 3.  Plane zz - 1 is complete
+// after input plane zz; its block is read, zeroed and taken by plane zz + 2.  Each output adds its
+// 27 taps in the same order and groups as in the row kernel (dz, then dy, then dx pairs), so
+// results are equal bit for bit.  A CTA's MMAs and epilogue alternate; the CTAs of an SM overlap
+// them.  128^3, 8 to 8 channels: 85 -> 33 us a launch (8 to 16: 90 -> 57); the prediction of the four-level
+// network 854 -> 631 us.  33 us is not the MMAs' time (13) but the steps' chain of load, MMAs,
+// accumulator read and store at two to three CTAs an SM (four hold less than they cost in runs).
+constexpr int kPlaneRows = 4;
+template <int CB>
+constexpr int kPlaneN = CB == 8 ? 32 : 48;  // accumulator columns of a row
+template <int CB, int G>
+constexpr uint32_t kPlaneB = 3 * (kPlaneN<CB> / 8) * (G == 1 ? 4 : 6) * 128;  // B of one zz mod 3: 3 rows, K cores
+constexpr uint32_t kPlaneLine = line_bytes(128), kPlaneBuf = (kPlaneRows + 2) * kPlaneLine, kPlaneGroup = 2 * kPlaneBuf;
+template <int CB, int G>
+constexpr size_t kPlaneSmem = 3 * kPlaneB<CB, G> + G * kPlaneGroup + 256;
+
+template <int CB, int G>
+__global__ void __launch_bounds__(kConvThreads) k_conv3_planes(Conv3Args a, int zrun, int runs) {
+  constexpr int W = 128, N = kPlaneN<CB>, kH = CB / 8, kCores = G == 1 ? 4 : 6;
+  constexpr uint32_t kB = kPlaneB<CB, G>;
+  constexpr uint32_t kCols = tmem_cols_for(kPlaneRows * N);
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t drain_bar;
+  __shared__ uint32_t tmem_slot;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const uint32_t sB = smem_u32(smem);
+  const uint32_t sL = sB + 3 * kB;
+  const int ny = a.d.ny, nz = a.d.nz;
+  const int chunks_y = (ny + kPlaneRows - 1) / kPlaneRows;
+  const int items = runs * chunks_y;
+
+  if (tid == 0) {
+    mbar_init(&bar, 1);
+    mbar_init(&drain_bar, 1);
+    fence_barrier_init();
+  }
+  if (warp == 0) tmem_alloc(&tmem_slot, kCols);
+  // Zeros: with 8 channels the third x offset's pair reads 16 bytes past its line under zero
+  // weights, and those bytes must be finite (as in the row kernel).
+  for (uint32_t off = (uint32_t)tid * 16; off < G * kPlaneGroup + 256; off += kConvThreads * 16)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sL + off), "r"(0u) : "memory");
+  // B of m = zz mod 3: N cores [row j: dy = 1 - j][block], K cores q of that dz and dy
+  for (uint32_t i = (uint32_t)tid; i < 3 * kB / 16; i += kConvThreads) {
+    const int n = i & 7, q = (i >> 3) % kCores, c = (int)(i >> 3) / kCores;
+    const int b = c % (N / 8), j = (c / (N / 8)) % 3, m = c / (3 * (N / 8));
+    const int zb = b / kH, dzi = zb == m ? 1 : (zb == (m + 1) % 3 ? 0 : 2);  // plane zb = zz - (dzi - 1) mod 3
+    const bool ok = zb < 3;
+    const bf16* w = a.w + (size_t)((b % kH) * 8 + n) * (9 * kCores * 8) + ((dzi * 3 + 2 - j) * kCores + q) * 8;
+    cp_async16(sB + i * 16, ok ? (const void*)w : (const void*)a.w, ok ? 16u : 0u);
+  }
+  cp_async_commit();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+  const uint32_t lane_t = tmem + ((uint32_t)(warp * 32) << 16);
+  const uint64_t adesc0 = G == 1 ? umma_sdesc(sL, 16, 128) : umma_sdesc(sL, kPlaneGroup, 128);
+  const uint64_t bdesc0 = umma_sdesc(sB, 128, kCores * 128);
+
+  // input plane zz exists (wrapped) or lies past a wall
+  auto plane_of = [&](int zz) { return zz >= 0 && zz < nz ? zz : (a.d.pz ? (zz < 0 ? zz + nz : zz - nz) : -1); };
+  // Loads: each thread takes its cell x = tid of every line, and threads 0 .. 12 G - 1 one halo
+  // cell (x = -1 or 128) of one line; offsets and the rows past a wall are found once an item.
+  constexpr int kLines = kPlaneRows + 2;
+  int l_off[kLines], l_size[kLines];
+  const bool halo = tid < 2 * kLines * G;
+  const int h_line = (tid >> 1) % kLines, h_cg = (tid >> 1) / kLines, h_side = tid & 1;
+  const uint32_t h_dst = sL + (uint32_t)h_cg * kPlaneGroup + (uint32_t)h_line * kPlaneLine + (h_side ? (W + 1) * 16u : 0u);
+  int h_off = 0, h_size = 0;
+  auto row_of = [&](int yy, bool& ok) {
+    ok = yy <= ny;
+    if (yy < 0 || yy == ny) {
+      if (a.d.py) yy = yy < 0 ? yy + ny : yy - ny;
+      else ok = false;
+    }
+    return ok ? yy : 0;
+  };
+  auto find_lines = [&](int y0) {
+#pragma unroll
+    for (int r = 0; r < kLines; ++r) {
+      bool ok;
+      const int yy = row_of(y0 - 1 + r, ok);
+      l_off[r] = (yy * W + tid) * a.ldx;
+      l_size[r] = ok ? 16 : 0;
+    }
+    bool ok;
+    const int yy = row_of(y0 - 1 + h_line, ok);
+    h_off = (yy * W + (h_side ? 0 : W - 1)) * a.ldx + h_cg * 8;  // x = W wraps to 0, x = -1 to W - 1
+    h_size = ok && a.d.px ? 16 : 0;
+  };
+  auto load_plane = [&](int zz, int buf) {
+    const int zw = plane_of(zz);
+    if (zw < 0) return;
+    const bf16* plane = a.x + (size_t)zw * ny * W * a.ldx;
+    const uint32_t dst = sL + (uint32_t)buf * kPlaneBuf + (uint32_t)(tid + 1) * 16;
+#pragma unroll
+    for (int r = 0; r < kLines; ++r) {
+      cp_async16(dst + (uint32_t)r * kPlaneLine, plane + l_off[r], (uint32_t)l_size[r]);
+      if (G == 2) cp_async16(dst + kPlaneGroup + (uint32_t)r * kPlaneLine, plane + l_off[r] + 8, (uint32_t)l_size[r]);
+    }
+    if (halo) cp_async16(h_dst + (uint32_t)buf * kPlaneBuf, plane + h_off, (uint32_t)h_size);
+  };
+
+  float bias_r[CB];
+#pragma unroll
+  for (int i = 0; i < CB; ++i) bias_r[i] = (a.bias && i < a.cout) ? __ldg(a.bias + i) : 0.0f;
+  int fail = 0;
+  uint32_t phase = 0;
+  for (int it = blockIdx.x; it < items && !fail; it += gridDim.x) {
+    const int run = it / chunks_y;
+    const int y0 = (it - run * chunks_y) * kPlaneRows;
+    const int rows = min(kPlaneRows, ny - y0);
+    const int z0 = run * zrun, z1 = min(nz, z0 + zrun);
+    for (int c = 0; c < kPlaneRows * N; c += 8) tmem_zero8(lane_t + (uint32_t)c);
+    tmem_st_wait();
+    find_lines(y0);
+    load_plane(z0 - 1, 0);
+    cp_async_commit();
+    for (int zz = z0 - 1; zz <= z1; ++zz) {
+      const int buf = (zz - z0 + 1) & 1;
+      const bool live = plane_of(zz) >= 0;
+      cp_async_wait<0>();  // plane zz (and the weights) have landed
+      fence_proxy_async();
+      tc_fence_before();  // this thread's reads and zeroes of the accumulators
+      fail = __syncthreads_or(fail);
+      if (fail) break;
+      if (warp == 0 && live && elect_one()) {
+        tc_fence_after();
+        const uint64_t b0 = bdesc0 + (uint64_t)((uint32_t)((zz + 3) % 3) * kB >> 4);
+        const uint64_t a0 = adesc0 + (uint64_t)(((uint32_t)buf * kPlaneBuf) >> 4);
+#pragma unroll
+        for (int l = 0; l < kLines; ++l) {  // line y0 - 1 + l: towards rows l - 2 .. l of the CTA's
+          constexpr int kStep = G == 1 ? 2 : 3;  // MMAs per line: x offsets (-1, 0) and (+1, none), or one each
+          const int lo = l < 2 ? 0 : l - 2, hi = l < kPlaneRows ? l : kPlaneRows - 1;
+          const uint32_t idesc = umma_idesc_bf16(W, (hi - lo + 1) * N, false, false);
+#pragma unroll
+          for (int h = 0; h < kStep; ++h)
+            umma_bf16(tmem + (uint32_t)(lo * N), a0 + (uint64_t)(((uint32_t)l * kPlaneLine + (G == 1 ? 32u : 16u) * h) >> 4),
+                      b0 + (uint64_t)((uint32_t)((lo - l + 2) * (N / 8) * kCores * 128 + h * 256) >> 4), idesc, 1u);
+        }
+        umma_commit(&bar);
+      }
+      if (zz < z1) load_plane(zz + 1, buf ^ 1);  // its buffer was read last by the MMAs of plane zz - 1
+      cp_async_commit();
+      // plane zz - 1 is complete after these MMAs: out, and its column block to plane zz + 2
+      const int z = zz - 1;
+      const uint32_t col = (uint32_t)(((z + 3) % 3) * CB);
+      const size_t v0 = ((size_t)max(z, 0) * ny + y0) * W + tid;
+      const bool keep = z >= z0;
+      uint4 mq[kPlaneRows * kH];
+      if (a.mask && keep) {  // read while the MMAs run
+#pragma unroll
+        for (int r = 0; r < kPlaneRows; ++r)
+#pragma unroll
+          for (int h = 0; h < kH; ++h)
+            if (r < rows && 8 * h < a.cout)
+              mq[r * kH + h] = *reinterpret_cast<const uint4*>(a.mask + (v0 + r * W) * a.ldm + 8 * h);
+      }
+      if (live) {
+        if (!mbar_wait(&bar, phase)) fail = 1;
+        phase ^= 1u;
+      }
+      tc_fence_after();
+      uint32_t acc[kPlaneRows * kH][8];
+#pragma unroll
+      for (int r = 0; r < kPlaneRows; ++r)
+#pragma unroll
+        for (int h = 0; h < kH; ++h) tmem_ld8_async(lane_t + (uint32_t)(r * N + 8 * h) + col, acc[r * kH + h]);
+      tmem_ld_wait(acc);
+#pragma unroll
+      for (int r = 0; r < kPlaneRows; ++r)
+#pragma unroll
+        for (int h = 0; h < kH; ++h) tmem_zero8(lane_t + (uint32_t)(r * N + 8 * h) + col);
+      if (keep && !fail) {
+#pragma unroll
+        for (int r = 0; r < kPlaneRows; ++r)
+#pragma unroll
+          for (int h = 0; h < kH; ++h) {
+            if (r >= rows || 8 * h >= a.cout) continue;
+            float o[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              float val = __uint_as_float(acc[r * kH + h][i]) + bias_r[8 * h + i];
+              if (a.relu) val = fmaxf(val, 0.0f);
+              o[i] = val;
+            }
+            if (a.mask) {
+              const bf16* mv = reinterpret_cast<const bf16*>(&mq[r * kH + h]);
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                if (!(__bfloat162float(mv[i]) > 0.0f)) o[i] = 0.0f;
+            }
+            uint4 q;
+            __nv_bfloat162* qp = reinterpret_cast<__nv_bfloat162*>(&q);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) qp[i] = __floats2bfloat162_rn(o[2 * i], o[2 * i + 1]);
+            *reinterpret_cast<uint4*>(a.y + (v0 + r * W) * a.ldy + 8 * h) = q;
+          }
+      }
+      tmem_st_wait();
+    }
+    fail = __syncthreads_or(fail);  // all of the CTA goes on, or none
+  }
+  cp_async_wait_all();
+  if (warp == 0 && elect_one()) {
+    umma_commit(&drain_bar);
+    if (!mbar_wait(&drain_bar, 0)) fail = 1;
+  }
+  if (fail && a.err) atomicExch(a.err, 1);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, kCols);
+}
+
 // ------------------------------------------- 3x3x3 convolution on slabs of short rows (MMA)
 //
 // Grids whose rows are short (W = 16, 32 or 64 cells: the network's coarser levels) take an
@@ -1994,7 +2221,42 @@ bool row_kernel_fits(const Dims& d, int cin, int np) {
          row_smem(np, cin, d.nx) <= kMaxConvSmem;
 }
 
+template <int CB, int G>
+rb_status launch_planes(const Conv3Args& a, cudaStream_t s) {
+  auto* kern = &k_conv3_planes<CB, G>;
+  constexpr size_t smem = kPlaneSmem<CB, G>;
+  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem));
+  thread_local int per_sm = 0;
+  if (per_sm == 0)
+    per_sm = blocks_per_sm(reinterpret_cast<const void*>(kern), smem, kConvThreads, tmem_cols_for(kPlaneRows * kPlaneN<CB>));
+  // Planes per run: two are read beyond the run's own, and the CTAs of an SM take turns (one alone
+  // idles while it waits: 1.8 times its share).  128^3, prediction by run length: 663 us at 4 or 5
+  // planes, 651 at 7, 641 at 10, 630 at 15 (this rule's), 642 at 19, 656 at 32.
+  const int sms = guess_sm_count(), chunks_y = (a.d.ny + kPlaneRows - 1) / kPlaneRows;
+  int zrun = 1;
+  double best = 1e30;
+  for (int l = 1; l <= a.d.nz; ++l) {
+    const int items = chunks_y * ((a.d.nz + l - 1) / l), on = (items + sms - 1) / sms;  // CTAs on the fullest SM
+    const int rounds = (on + per_sm - 1) / per_sm;
+    const double cost = (l + 2) * std::max((double)on, 1.8 * rounds);
+    if (cost < best) best = cost, zrun = l;
+  }
+  const int runs = (a.d.nz + zrun - 1) / zrun;
+  const int grid = std::max(1, std::min(runs * chunks_y, per_sm * sms));
+  kern<<<grid, kConvThreads, smem, s>>>(a, zrun, runs);
+  RB_CUDA(cudaGetLastError());
+  return RB_OK;
+}
+
+// rows of 128 cells, 8 or 16 input channels and at most 16 output channels: more of either and the
+// three copies of B and the lines leave one CTA per SM (the row kernel holds one copy)
+bool planes_fit(const Dims& d, int cin, int cout) { return d.nx == 128 && (cin == 8 || cin == 16) && cout <= 16; }
+
 rb_status row_launch(const Conv3Args& a, int np, cudaStream_t s) {
+  if (planes_fit(a.d, a.cin, a.cout)) {
+    if (a.cin == 8) return a.cout <= 8 ? launch_planes<8, 1>(a, s) : launch_planes<16, 1>(a, s);
+    return a.cout <= 8 ? launch_planes<8, 2>(a, s) : launch_planes<16, 2>(a, s);
+  }
   const size_t smem = row_smem(np, a.cin, a.d.nx);
   const bool w128 = a.d.nx == 128;
   switch (np) {

@@ -32,6 +32,16 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N, bool a_mn, 
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// One lane of a converged warp, the same one every time.  MMAs issued under it (in a branch on a
+// warp index that __shfl_sync made uniform) keep their descriptors in uniform registers: 40 cycles
+// an MMA of N <= 32 unrolled, the tensor pipe's own rate (32 + N / 4 cycles, whatever the layout),
+// where a branch on threadIdx.x takes 46 unrolled and 83 in a loop.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+  return p != 0;
+}
+
 // D[tmem] (+)= A * B^T for one K = 16 step; issued by a single thread.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           uint32_t accumulate) {
@@ -77,6 +87,27 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+
+// Whole warp: 8 consecutive FP32 columns of a TMEM lane, read (the values are there after
+// tmem_ld_wait) or set to zero (tmem_st_wait before the columns are used again).
+__device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+template <int M>
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[M][8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < M; ++i)  // no use of the values moves above the wait
+#pragma unroll
+    for (int j = 0; j < 8; ++j) asm volatile("" : "+r"(r[i][j]));
+}
+__device__ __forceinline__ void tmem_zero8(uint32_t taddr) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr), "r"(0u) : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 16-byte asynchronous global -> shared copy; `bytes` = 16 copies, 0 writes zeros.
 __device__ __forceinline__ void cp_async16(uint32_t sdst, const void* gsrc, uint32_t bytes) {
