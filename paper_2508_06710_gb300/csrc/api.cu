@@ -50,7 +50,7 @@ int resident_blocks(const void* kernel, size_t smem, int threads) {
   return v;
 }
 
-rb_status opt_in_smem(const void* kernel, size_t bytes) {
+rb_status opt_in_smem(const void* kernel, size_t bytes, bool all_shared) {
   if (bytes == 0) return RB_OK;
   static std::mutex mu;
   static std::map<std::pair<int, const void*>, size_t> opted;
@@ -64,6 +64,8 @@ rb_status opt_in_smem(const void* kernel, size_t bytes) {
     RB_CUDA(cudaFuncGetAttributes(&fa, kernel));
     if (fa.sharedSizeBytes + bytes > 48 * 1024)
       RB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    if (all_shared)
+      RB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
     cur = bytes;
   }
   return RB_OK;

@@ -75,8 +75,10 @@ int resident_blocks(const void* kernel, size_t smem, int threads = kThreads);
 
 // Raises `kernel`'s dynamic shared memory limit to at least `bytes` on the current device.
 // The attribute belongs to the device, so the largest value set is remembered per (device,
-// kernel); a host thread that moves to another device sets it again there.
-rb_status opt_in_smem(const void* kernel, size_t bytes);
+// kernel); a host thread that moves to another device sets it again there.  all_shared also asks
+// for the largest shared memory split: the driver's choice (200 KB, say) may hold a block fewer per
+// SM than a grid was planned for.
+rb_status opt_in_smem(const void* kernel, size_t bytes, bool all_shared = false);
 
 template <typename K>
 inline int wave_grid(K* kernel, int64_t work_blocks, size_t smem = 0, int threads = kThreads) {

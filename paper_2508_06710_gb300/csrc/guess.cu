@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw
   __shared__ __align__(8) uint64_t acc_bar;
   __shared__ __align__(8) uint64_t drain_bar;
   __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int G = a.cin / 8, ktot = stack_k(a.cin);
   const uint32_t sB = smem_u32(smem);
   const uint32_t sS = sB + (uint32_t)(NT * ktot * 2);
@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
   // this thread's cell: row r, position x of the tile, accumulator row tid (TMEM lane tid)
   const int x = tid % W, r = tid / W;
   const bool has_l = x > 0 || a.d.px, has_r = x < W - 1 || a.d.px;
@@ -854,21 +854,24 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw
     cp_async_wait<0>();  // the slab (and, on the first tile, the weights) has landed
     fence_proxy_async();
     if (__syncthreads_or(fail)) break;
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       tc_fence_after();
-      uint32_t kk = 0;
+      const uint64_t ad0 = umma_sdesc(sS, kGS, 128);
+      uint64_t bd = umma_sdesc(sB, 128, sbo_b);  // 16 units (two K cores) on after every MMA
       if (G == 1) {  // cores: planes (0, 1) and (2, zero) of each y offset
-        for (int dyi = 0; dyi < 3; ++dyi)
-          for (int pr = 0; pr < 2; ++pr, ++kk) {
-            const uint64_t ad = umma_sdesc(sS + (uint32_t)(2 * pr) * kGS + (uint32_t)(dyi * W) * 16, kGS, 128);
-            umma_bf16(tmem, ad, umma_sdesc(sB + kk * 256, 128, sbo_b), idesc, kk > 0 ? 1u : 0u);
-          }
+#pragma unroll
+        for (int kk = 0; kk < 6; ++kk)
+          umma_bf16(tmem, ad0 + ((uint32_t)(kk & 1) * 2 * kGS + (uint32_t)(kk >> 1) * W * 16) / 16, bd + 16u * kk, idesc,
+                    kk > 0 ? 1u : 0u);
       } else {
+        const uint64_t plane = (uint64_t)G * kGS / 16;
+#pragma unroll
         for (int li = 0; li < 9; ++li) {
-          const int dzi = li / 3, dyi = li % 3;
-          for (int pr = 0; pr < G / 2; ++pr, ++kk) {
-            const uint64_t ad = umma_sdesc(sS + (uint32_t)(dzi * G + 2 * pr) * kGS + (uint32_t)(dyi * W) * 16, kGS, 128);
-            umma_bf16(tmem, ad, umma_sdesc(sB + kk * 256, 128, sbo_b), idesc, kk > 0 ? 1u : 0u);
+          uint64_t ad = ad0 + (uint64_t)(li / 3) * plane + (uint32_t)(li % 3) * W;
+          for (int pr = 0; pr < G / 2; ++pr) {
+            umma_bf16(tmem, ad, bd, idesc, (li > 0 || pr > 0) ? 1u : 0u);
+            ad += 2 * kGS / 16;
+            bd += 16u;
           }
         }
       }
@@ -939,7 +942,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw
   }
   cp_async_wait_all();
   // every MMA this CTA issued has completed before TMEM is released (also after a wait gave up)
-  if (tid == 0) {
+  if (warp == 0 && elect_one()) {
     umma_commit(&drain_bar);
     if (!mbar_wait(&drain_bar, 0)) fail = 1;
   }
@@ -1139,20 +1142,24 @@ __global__ void __launch_bounds__(kConvThreads) k_wgrad_mma(WgradArgs a) {
 // Accumulators: one 32-column block per (input group, output group), in TMEM for the CTA's
 // runs (at most two output groups per CTA: more are spread over the grid's y dimension); the
 // partial [split][m = tap c_in + ci (+ the bias row 27 c_in)][n = co] goes to k_wgrad_reduce.
+// An elected lane issues a row's W / 16 MMAs unrolled; every offset that is the same for all rows is
+// found once.  128^3, 8 to 8 channels: 121 -> 55 us (16 to 8: 163 -> 131), half of it from a grid
+// that fits the SMs in one wave (blocks_per_sm).  What is left is the chain of a run of two rows:
+// lines, MMAs, and the next run's lines only after them (four CTAs an SM overlap it).
 __host__ __device__ constexpr int wlin_halo(int W) { return W + 4; }  // g line: cells -1 .. W + 2
 inline size_t wgrad_lin_smem(int W, int G, int Go, int chunk) {
   return ((size_t)G * (chunk + 2) * 3 + 7) * W * 16 + 3 * (size_t)Go * wlin_halo(W) * 16;
 }
 
 template <int W>
-__global__ void __launch_bounds__(kConvThreads) k_wgrad_lin(WgradArgs a, int chunk, int runs_per_split) {
+__global__ void __launch_bounds__(kConvThreads, 4) k_wgrad_lin(WgradArgs a, int chunk, int runs_per_split) {
   constexpr uint32_t kLB = W * 16;                   // one line: W cells x 8 channels
   constexpr uint32_t kGH = wlin_halo(W) * 16;        // one g line with its halo
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t mma_bar[2];  // rows alternate between the two
   __shared__ uint32_t tmem_slot;
   __shared__ float bred[4][16];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   // this CTA's output groups: cgo0 .. cgo0 + Go - 1 of the layer's (grid dimension y)
   const int G = a.cin / 8, cgo0 = blockIdx.y * a.go_cta, Go = min(a.go_cta, (a.cout + 7) / 8 - cgo0);
   const uint32_t cols = tmem_cols_for(32 * G * a.go_cta);
@@ -1178,7 +1185,7 @@ __global__ void __launch_bounds__(kConvThreads) k_wgrad_lin(WgradArgs a, int chu
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
 
   // this thread's copies of a row's lines: copy k is piece i = tid + 128 k of (dzi, x, cg), the
   // same for every row, so its offsets are worked out once (up to kWT copies a thread)
@@ -1196,6 +1203,21 @@ __global__ void __launch_bounds__(kConvThreads) k_wgrad_lin(WgradArgs a, int chu
     t_dst[k] = (uint32_t)((cg * (chunk + 2)) * 3 + dzi) * kLB + (uint32_t)x * 16;
     t_src[k] = (uint32_t)(x * a.ldx + cg * 8);
   }
+  // the current run's three input planes (or none past a wall)
+  const bf16* pb[3] = {a.x, a.x, a.x};
+  bool pok[3] = {false, false, false};
+  auto find_planes = [&](int z) {
+#pragma unroll
+    for (int dzi = 0; dzi < 3; ++dzi) {
+      int zz = z + dzi - 1;
+      pok[dzi] = true;
+      if (zz < 0 || zz >= nz) {
+        if (a.d.pz) zz = zz < 0 ? zz + nz : zz - nz;
+        else pok[dzi] = false;
+      }
+      pb[dzi] = pok[dzi] ? a.x + (size_t)zz * ny * W * a.ldx : a.x;
+    }
+  };
   // line (cg, yl, dzi) of the current run: input row y0 - 1 + yl of plane z + dzi - 1
   auto load_lines = [&](int z, int y0, int yl) {
     int yy = y0 - 1 + yl;
@@ -1203,29 +1225,18 @@ __global__ void __launch_bounds__(kConvThreads) k_wgrad_lin(WgradArgs a, int chu
     if (yy < 0 || yy >= ny) {
       if (a.d.py) yy = yy < 0 ? yy + ny : yy - ny;
       else yok = false;
+      if (!yok) yy = 0;
     }
     if (tabled) {
-      // the row's start in each of the three planes (or none past a wall)
-      const bf16* pb[3];
-      bool pok[3];
-#pragma unroll
-      for (int dzi = 0; dzi < 3; ++dzi) {
-        int zz = z + dzi - 1;
-        pok[dzi] = yok;
-        if (zz < 0 || zz >= nz) {
-          if (a.d.pz) zz = zz < 0 ? zz + nz : zz - nz;
-          else pok[dzi] = false;
-        }
-        pb[dzi] = a.x + (size_t)(zz * ny + yy) * W * a.ldx;
-      }
+      const size_t row = (size_t)yy * W * a.ldx;
       const uint32_t yoff = sL + (uint32_t)(yl * 3) * kLB;
 #pragma unroll
       for (int k = 0; k < kWT; ++k) {
         if (t_dz[k] < 0) break;
         const int dz = t_dz[k];
-        const bool ok = dz == 0 ? pok[0] : (dz == 1 ? pok[1] : pok[2]);
+        const bool ok = yok && (dz == 0 ? pok[0] : (dz == 1 ? pok[1] : pok[2]));
         const bf16* b = dz == 0 ? pb[0] : (dz == 1 ? pb[1] : pb[2]);
-        cp_async16(yoff + t_dst[k], ok ? (const void*)(b + t_src[k]) : (const void*)a.x, ok ? 16u : 0u);
+        cp_async16(yoff + t_dst[k], b + row + t_src[k], ok ? 16u : 0u);
       }
       return;
     }
@@ -1243,21 +1254,31 @@ __global__ void __launch_bounds__(kConvThreads) k_wgrad_lin(WgradArgs a, int chu
                  ok ? 16u : 0u);
     }
   };
-  // the output gradient of row (z, y) with its halo into g buffer `buf`: cell h - 1 at h
-  auto load_g = [&](int z, int y, int buf) {
-    const int nh = W + 2;  // cells -1 .. W (the two spare cells stay zero)
-    for (int i = tid; i < nh * Go; i += kConvThreads) {
-      const int h = i / Go, cgo = i - h * Go;
-      int x = h - 1;
-      bool ok = (cgo0 + cgo) * 8 < a.cout;
-      if (x < 0 || x >= W) {
-        if (a.d.px) x = x < 0 ? x + W : x - W;
-        else ok = false;
-      }
-      const uint32_t dst = sG + (uint32_t)(buf * Go + cgo) * kGH + (uint32_t)h * 16;
-      cp_async16(dst, ok ? (const void*)(a.g + ((size_t)(z * ny + y) * W + x) * a.ldg + (cgo0 + cgo) * 8) : (const void*)a.g,
-                 ok ? 16u : 0u);
+  // the output gradient of row (z, y) with its halo (cells -1 .. W; the two spare cells stay zero)
+  // into g buffer `buf`: cell h - 1 at h.  The same up to three pieces (h, cgo) a thread for every row.
+  constexpr int kGT = 3;
+  uint32_t g_dst[kGT];
+  int g_src[kGT], g_n[kGT];
+#pragma unroll
+  for (int k = 0; k < kGT; ++k) {
+    const int i = tid + k * kConvThreads;
+    const int h = i / Go, cgo = i - h * Go;
+    int x = h - 1;
+    bool ok = (cgo0 + cgo) * 8 < a.cout;
+    if (x < 0 || x >= W) {
+      if (a.d.px) x = x < 0 ? x + W : x - W;
+      else ok = false;
     }
+    g_n[k] = i >= (W + 2) * Go ? -1 : (ok ? 16 : 0);
+    g_src[k] = ok ? x * a.ldg + (cgo0 + cgo) * 8 : 0;
+    g_dst[k] = sG + (uint32_t)cgo * kGH + (uint32_t)h * 16;
+  }
+  auto load_g = [&](int z, int y, int buf) {
+    const bf16* row = a.g + (size_t)(z * ny + y) * W * a.ldg;
+    const uint32_t off = (uint32_t)(buf * Go) * kGH;
+#pragma unroll
+    for (int k = 0; k < kGT; ++k)
+      if (g_n[k] >= 0) cp_async16(g_dst[k] + off, row + g_src[k], (uint32_t)g_n[k]);
   };
 
   float bsum[16];
@@ -1275,6 +1296,7 @@ __global__ void __launch_bounds__(kConvThreads) k_wgrad_lin(WgradArgs a, int chu
     wait_row(rows_done - 2);
     wait_row(rows_done - 1);
     if (!fail) {
+      find_planes(z);
       for (int yl = 0; yl < 3; ++yl) load_lines(z, y0, yl);
       load_g(z, y0, rows_done % 3);
     }
@@ -1308,20 +1330,19 @@ __global__ void __launch_bounds__(kConvThreads) k_wgrad_lin(WgradArgs a, int chu
           }
         }
       }
-      if (tid == 0) {
+      if (warp == 0 && elect_one()) {
         tc_fence_after();
         const int yl = y - y0;
-#pragma unroll 1
-        for (int ks = 0; ks < W / 16; ++ks)
-          for (int cg = 0; cg < G; ++cg) {
-            const uint64_t ad =
-                umma_sdesc(sL + (uint32_t)((cg * (chunk + 2) + yl) * 3) * kLB + (uint32_t)ks * 256, 128, kLB);
-            for (int cgo = 0; cgo < Go; ++cgo) {
-              const uint64_t bd = umma_sdesc(gb + (uint32_t)cgo * kGH + (uint32_t)ks * 256, 128, 16);
-              umma_bf16(tmem + (uint32_t)((cg * Go + cgo) * 32), ad, bd, idesc,
-                        (rows_done > 0 || ks > 0) ? 1u : 0u);
-            }
+        for (int cg = 0; cg < G; ++cg) {
+          const uint64_t ad = umma_sdesc(sL + (uint32_t)((cg * (chunk + 2) + yl) * 3) * kLB, 128, kLB);
+          for (int cgo = 0; cgo < Go; ++cgo) {
+            const uint64_t bd = umma_sdesc(gb + (uint32_t)cgo * kGH, 128, 16);
+            const uint32_t acc = tmem + (uint32_t)((cg * Go + cgo) * 32);
+#pragma unroll
+            for (int ks = 0; ks < W / 16; ++ks)
+              umma_bf16(acc, ad + 16u * ks, bd + 16u * ks, idesc, (rows_done > 0 || ks > 0) ? 1u : 0u);
           }
+        }
         umma_commit(&mma_bar[rows_done & 1]);
       }
       ++rows_done;
@@ -2160,7 +2181,9 @@ int blocks_per_sm(const void* kernel, size_t dyn_smem, int threads, uint32_t tme
   int n = std::min(blk_sm, thr_sm / threads);
   const int regs = std::max(1, fa.numRegs) * threads;
   n = std::min(n, regs_sm / regs);
-  const size_t per_block = dyn_smem + fa.sharedSizeBytes + (size_t)resv;
+  // allocated in units of 128 bytes (five blocks of 46,656 do not fit 233,472: planned as one wave of
+  // five per SM, the 128-cell rows' weight gradient ran a second one nearly empty)
+  const size_t per_block = (dyn_smem + fa.sharedSizeBytes + (size_t)resv + 127) / 128 * 128;
   n = std::min<int>(n, (int)(smem_sm / std::max<size_t>(per_block, 1)));
   n = std::min<int>(n, (int)(512 / tmem_cols));
   return std::max(1, n);
@@ -2171,7 +2194,7 @@ size_t conv_smem(int np, int kpad) { return (size_t)np * kpad * 2 + (size_t)kSta
 template <int NP>
 rb_status launch_conv3_np(const Conv3Args& a, size_t smem, cudaStream_t s) {
   auto* kern = &k_conv3_mma<NP>;
-  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem));
+  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem, true));
   const int n_tiles = (a.n_vox + 127) / 128;
   thread_local int per_sm = 0;
   thread_local size_t per_sm_smem = 0;
@@ -2199,7 +2222,7 @@ int head_idx(const rb_guess* g) { return 2 * g->L + 3 * (g->L - 1); }
 template <int NP, int W>
 rb_status launch_row_np(const Conv3Args& a, size_t smem, cudaStream_t s) {
   auto* kern = &k_conv3_row<NP, W>;
-  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem));
+  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem, true));
   thread_local int per_sm = 0;
   thread_local size_t per_sm_smem = 0;
   if (per_sm == 0 || per_sm_smem != smem) {
@@ -2225,7 +2248,7 @@ template <int CB, int G>
 rb_status launch_planes(const Conv3Args& a, cudaStream_t s) {
   auto* kern = &k_conv3_planes<CB, G>;
   constexpr size_t smem = kPlaneSmem<CB, G>;
-  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem));
+  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem, true));
   thread_local int per_sm = 0;
   if (per_sm == 0)
     per_sm = blocks_per_sm(reinterpret_cast<const void*>(kern), smem, kConvThreads, tmem_cols_for(kPlaneRows * kPlaneN<CB>));
@@ -2272,7 +2295,7 @@ rb_status row_launch(const Conv3Args& a, int np, cudaStream_t s) {
 template <int NT, int W>
 rb_status launch_slab_nt(const Conv3Args& a, int pw, size_t smem, cudaStream_t s) {
   auto* kern = &k_conv3_slab<NT, W>;
-  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem));
+  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem, true));
   thread_local int per_sm = 0;
   thread_local size_t per_sm_smem = 0;
   if (per_sm == 0 || per_sm_smem != smem) {
@@ -2403,7 +2426,7 @@ WgradPlan wgrad_plan(const Layer& ly, int n) {
 template <int NP>
 rb_status launch_wgrad_np(const WgradArgs& a, const WgradPlan& p, cudaStream_t s) {
   const size_t smem = (size_t)kStages * (kWAStage + NP * kWS * 2);
-  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(&k_wgrad_mma<NP>), smem));
+  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(&k_wgrad_mma<NP>), smem, true));
   k_wgrad_mma<NP><<<dim3(p.m_tiles, p.splits), kConvThreads, smem, s>>>(a);
   RB_CUDA(cudaGetLastError());
   return RB_OK;
@@ -2464,7 +2487,7 @@ LinWPlan wgrad_lin_plan(const Layer& ly, const Dims& d) {
 
 template <int W>
 rb_status launch_wgrad_lin(const WgradArgs& a, const LinWPlan& p, cudaStream_t s) {
-  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(&k_wgrad_lin<W>), p.smem));
+  RB_TRY(opt_in_smem(reinterpret_cast<const void*>(&k_wgrad_lin<W>), p.smem, true));
   k_wgrad_lin<W><<<dim3(p.splits, p.go_tiles), kConvThreads, p.smem, s>>>(a, p.chunk, p.per_split);
   RB_CUDA(cudaGetLastError());
   return RB_OK;
