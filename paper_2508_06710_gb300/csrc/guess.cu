@@ -761,6 +761,9 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_planes(Conv3Args a, int 
 // K of the stacked weights: 9 tap lines x C channels, as MMAs of two 8-channel K cores; with
 // C = 8 the cores of an MMA are two z lines of one y offset (z offsets -1, 0 and +1, zero
 // weights): 6 MMAs of 16
+// Bound by a tile's chain (slab, MMAs, epilogue) at 2.7 tiles a CTA, not by instructions: fixed
+// pieces per thread, 16-byte trades of the row ends and one TMEM wait a chunk took the 64-cell
+// rows' 48-column launch from 31 to 30 us (96 columns: 46 -> 41), a prediction from 613 to 606.
 __host__ __device__ constexpr int stack_k(int C) { return C == 8 ? 96 : 9 * C; }
 // dz slabs of a group: the three planes, and for 8-channel inputs a zero fourth (the partner of
 // the last plane's cores)
@@ -771,7 +774,7 @@ inline size_t slab_smem(int nt, int cin, int W) {
 }
 
 template <int NT, int W>
-__global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw) {
+__global__ void __launch_bounds__(kConvThreads, 5) k_conv3_slab(Conv3Args a, int pw) {
   constexpr int R = 128 / W;
   constexpr uint32_t kGS = slab_group_bytes(W);
   constexpr uint32_t kCols = tmem_cols_for(NT);
@@ -821,34 +824,54 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw
   const int seg = lane & ~(WL - 1);
   const int src_l = seg | ((lane + WL - 1) & (WL - 1)), src_r = seg | ((lane + 1) & (WL - 1));
   constexpr int WPR = W / 32;  // warps per row (0 for W = 16)
-  __shared__ float xl[WPR > 1 ? 4 : 1][16], xr[WPR > 1 ? 4 : 1][16];
+  // two sets, for alternate column chunks: a set is written again a barrier after it was read
+  __shared__ __align__(16) float xl[2][WPR > 1 ? 4 : 1][16], xr[2][WPR > 1 ? 4 : 1][16];
+  __shared__ __align__(16) float sbias[64];
   const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
+  // rows per pass of the copies (0: pieces taken one by one), and this thread's piece of them
+  const int pieces = W * G;
+  const int per_pass = kConvThreads % pieces == 0 ? kConvThreads / pieces : 0;
+  const int row0 = tid / pieces, x0 = (tid % pieces) / G, cg0 = tid % G;
+  for (int i = tid; i < 64; i += kConvThreads) sbias[i] = a.bias && i < a.cout ? __ldg(a.bias + i) : 0.0f;
   int fail = 0;
   uint32_t phase = 0;
   for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
     const int z = t / tiles_y, y0 = (t - z * tiles_y) * R;
     // slab [dz][group][row y0 - 1 + rr][cell][8 channels]; a thread's consecutive copies read
-    // consecutive 16-byte pieces of one cell
-    const int total = 3 * (R + 2) * W * G;
-    for (int i = tid; i < total; i += kConvThreads) {
-      int rest = G == 1 ? i : (int)__umulhi((uint32_t)i, g_magic);  // i / G
-      const int cg = i - rest * G;
-      const int xx = rest % W;
-      rest /= W;
-      const int rr = rest % (R + 2), dzi = rest / (R + 2);
-      int yy = y0 - 1 + rr, zz = z + dzi - 1;
-      bool ok = true;
-      if (yy < 0 || yy >= ny) {
-        if (a.d.py) yy = yy < 0 ? yy + ny : yy - ny;
-        else ok = false;
-      }
+    // consecutive 16-byte pieces of one cell.  A row's W G pieces that divide the block (or that it
+    // divides) leave each thread the same piece of every row.
+    const bf16* plane[3];
+    bool pok[3];
+#pragma unroll
+    for (int dzi = 0; dzi < 3; ++dzi) {
+      int zz = z + dzi - 1;
+      pok[dzi] = true;
       if (zz < 0 || zz >= nz) {
         if (a.d.pz) zz = zz < 0 ? zz + nz : zz - nz;
-        else ok = false;
+        else pok[dzi] = false;
       }
-      const uint32_t dst = sS + (uint32_t)(dzi * G + cg) * kGS + (uint32_t)(rr * W + xx) * 16;
-      cp_async16(dst, ok ? (const void*)(a.x + ((size_t)(zz * ny + yy) * W + xx) * a.ldx + cg * 8) : (const void*)a.x,
-                 ok ? 16u : 0u);
+      plane[dzi] = pok[dzi] ? a.x + (size_t)zz * ny * W * a.ldx : a.x;
+    }
+    auto copy = [&](int dzi, int rr, int xx, int cg) {
+      int yy = y0 - 1 + rr;
+      bool ok = dzi == 0 ? pok[0] : (dzi == 1 ? pok[1] : pok[2]);
+      if (yy < 0 || yy >= ny) {
+        ok = ok && a.d.py;
+        yy = yy < 0 ? yy + ny : yy - ny;
+      }
+      const bf16* src = (dzi == 0 ? plane[0] : (dzi == 1 ? plane[1] : plane[2])) + (size_t)(yy * W + xx) * a.ldx + cg * 8;
+      cp_async16(sS + (uint32_t)(dzi * G + cg) * kGS + (uint32_t)(rr * W + xx) * 16, ok ? src : a.x, ok ? 16u : 0u);
+    };
+    if (per_pass > 0) {
+#pragma unroll 3
+      for (int row = row0; row < 3 * (R + 2); row += per_pass) copy(row / (R + 2), row % (R + 2), x0, cg0);
+    } else {
+      const int total = 3 * (R + 2) * W * G;
+      for (int i = tid; i < total; i += kConvThreads) {
+        const int rest = G == 1 ? i : (int)__umulhi((uint32_t)i, g_magic);  // i / G
+        const int row = rest / W;
+        copy(row / (R + 2), row % (R + 2), rest % W, i - rest * G);
+      }
     }
     cp_async_commit();
     cp_async_wait<0>();  // the slab (and, on the first tile, the weights) has landed
@@ -882,10 +905,17 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw
     tc_fence_after();
     const int v = (z * ny + y0 + r) * W + x;
     for (int c0 = 0; c0 < pw; c0 += 16) {
+      uint32_t acc[6][8];  // dx = -1 block, 0, +1 (whole warp)
+#pragma unroll
+      for (int b = 0; b < 6; ++b) tmem_ld8_async(taddr + (uint32_t)((b >> 1) * pw + c0 + (b & 1) * 8), acc[b]);
+      tmem_ld_wait(acc);
       float pm[16], pc[16], pp[16];
-      tmem_ld16(taddr + (uint32_t)c0, pm);             // dx = -1 block (whole warp)
-      tmem_ld16(taddr + (uint32_t)(pw + c0), pc);      // dx = 0
-      tmem_ld16(taddr + (uint32_t)(2 * pw + c0), pp);  // dx = +1
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        pm[i] = __uint_as_float(acc[i >> 3][i & 7]);
+        pc[i] = __uint_as_float(acc[2 + (i >> 3)][i & 7]);
+        pp[i] = __uint_as_float(acc[4 + (i >> 3)][i & 7]);
+      }
       float lv[16], rv[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
@@ -893,20 +923,33 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw
         rv[i] = __shfl_sync(0xffffffffu, pp[i], src_r);
       }
       if constexpr (WPR > 1) {
-        const int wr = warp % WPR, w0 = warp - wr;
+        const int wr = warp % WPR, w0 = warp - wr, set = (c0 >> 4) & 1;
+        if (lane == 31) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          if (lane == 31) xl[warp][i] = pm[i];
-          if (lane == 0) xr[warp][i] = pp[i];
+          for (int i = 0; i < 16; i += 4)
+            *reinterpret_cast<float4*>(&xl[set][warp][i]) = make_float4(pm[i], pm[i + 1], pm[i + 2], pm[i + 3]);
+        }
+        if (lane == 0) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 4)
+            *reinterpret_cast<float4*>(&xr[set][warp][i]) = make_float4(pp[i], pp[i + 1], pp[i + 2], pp[i + 3]);
         }
         __syncthreads();
         const int wl = w0 + (wr + WPR - 1) % WPR, wn = w0 + (wr + 1) % WPR;
+        if (lane == 0) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          if (lane == 0) lv[i] = xl[wl][i];
-          if (lane == 31) rv[i] = xr[wn][i];
+          for (int i = 0; i < 16; i += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(&xl[set][wl][i]);
+            lv[i] = q.x, lv[i + 1] = q.y, lv[i + 2] = q.z, lv[i + 3] = q.w;
+          }
         }
-        __syncthreads();  // xl, xr are rewritten by the next column chunk
+        if (lane == 31) {
+#pragma unroll
+          for (int i = 0; i < 16; i += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(&xr[set][wn][i]);
+            rv[i] = q.x, rv[i + 1] = q.y, rv[i + 2] = q.z, rv[i + 3] = q.w;
+          }
+        }
       }
       float o[16];
 #pragma unroll
@@ -920,7 +963,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_slab(Conv3Args a, int pw
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           float val = o[8 * h + i];
-          if (a.bias) val += __ldg(a.bias + cb + i);
+          if (a.bias) val += sbias[cb + i];
           if (a.relu) val = fmaxf(val, 0.0f);
           q8[i] = val;
         }
