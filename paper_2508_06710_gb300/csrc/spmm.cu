@@ -61,7 +61,7 @@ std::vector<int> vec_candidates(int eb, int k) {
 // extruded mesh):
 //   long rows (12 to 40 entries: the 13- and 27-point operators').  FP32: the TMA ring, whose entries
 //     come from shared memory while eight or more gathers per lane are in flight (27p k = 1, 3, 8
-//     137, 163, 211 and with the row split over lanes 185, 224, 353; 13p k = 1, 3 74, 86 and 91, 107;
+//     137, 163, 216 and with the row split over lanes 185, 224, 353; 13p k = 1, 3 74, 86 and 91, 107;
 //     not 13p k = 8, 140 and direct 134; 27p k = 4 in halves, 164 against 168).  FP64 is
 //     bound by its pipe and splitting a row pays shuffles on it: one lane per row, in the ring where
 //     loads still matter (27p k = 1, 2, 3 239, 380, 570 and direct 291, 397, 662; 13p k = 1 109 and

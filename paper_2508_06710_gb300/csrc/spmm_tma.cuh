@@ -24,7 +24,7 @@ namespace rb {
 // rows (LONG): a tile is tens of KB, so two stages and as many consumers as keep a tile near 28 KB
 // (four blocks per SM), and each lane issues kLongGathers gathers before it uses the first: a row's
 // gathers are an L2 round trip each, and two at a time left the 16 resident consumer warps waiting.
-// 160^3 27-point operator, FP32 k = 8: 211 us (1.16 GB: 0.82 of the measured HBM rate; three blocks
+// 160^3 27-point operator, FP32 k = 8: 216 us (1.16 GB: 0.80 of the measured HBM rate; three blocks
 // per SM, left to itself the compiler fits two: 254); with three stages 347, two gathers at a time
 // over 380, direct with eight threads a row 353; 13-point, k = 4: 90 us against 105 (direct).
 template <bool LONG>
@@ -179,29 +179,33 @@ __global__ void __launch_bounds__(kTmaThreads, LONG ? (sizeof(T) == 4 ? 3 : 2) :
       const T* Xc = a.X + chunk * VEC;
       if (staged) {
         int p = rs;
+        T sum[LONG ? VEC : 1] = {};  // of an FP32 row's batches; the rest of the row sums in acc
         if constexpr (LONG) {
-          // FP32: two running sums, for a smaller rounding error than one; FP64: one (a further
-          // addition would take a slot of its pipe)
-          constexpr int U = kLongGathers<T, VEC>, A = sizeof(T) == 4 ? 2 : 1;
-          T part[A][VEC];
-#pragma unroll
-          for (int q = 0; q < A; ++q)
-#pragma unroll
-            for (int ee = 0; ee < VEC; ++ee) part[q][ee] = T(0);
+          // FP32: a batch sums in four chains of its own, and its sum joins the row's, so rounding
+          // grows with the batches and not with the entries (27p k = 8, against 64 bits: 6.7e-8, as with
+          // the row split over lanes; one pair of chains through the row 8.3e-8 in 211 us).  FP64: one chain (a further addition
+          // takes a slot of its pipe).
+          constexpr int U = kLongGathers<T, VEC>, A = sizeof(T) == 4 ? 4 : 1;
           for (; p + U <= re; p += U) {
             Vec<T, VEC> x[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) x[u] = ldv<T, VEC>(Xc + (int64_t)s_ci[p + u] * a.ldx);
+            T part[A][VEC];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
               const T v = s_va[p + u];
 #pragma unroll
-              for (int ee = 0; ee < VEC; ++ee) part[u % A][ee] = fma(v, x[u].v[ee], part[u % A][ee]);
+              for (int ee = 0; ee < VEC; ++ee) {
+                if constexpr (A == 1) acc[ee] = fma(v, x[u].v[ee], acc[ee]);
+                else part[u % A][ee] = u < A ? v * x[u].v[ee] : fma(v, x[u].v[ee], part[u % A][ee]);
+              }
+            }
+            if constexpr (A == 4) {
+#pragma unroll
+              for (int ee = 0; ee < VEC; ++ee)
+                sum[ee] += (part[0][ee] + part[1][ee]) + (part[2][ee] + part[3][ee]);
             }
           }
-#pragma unroll
-          for (int ee = 0; ee < VEC; ++ee)
-            acc[ee] = A == 2 ? part[0][ee] + part[1 % A][ee] : part[0][ee];
         }
 #pragma unroll 2
         for (; p < re; ++p) {
@@ -210,6 +214,10 @@ __global__ void __launch_bounds__(kTmaThreads, LONG ? (sizeof(T) == 4 ? 3 : 2) :
           const Vec<T, VEC> x = ldv<T, VEC>(Xc + (int64_t)c * a.ldx);
 #pragma unroll
           for (int ee = 0; ee < VEC; ++ee) acc[ee] = fma(v, x.v[ee], acc[ee]);
+        }
+        if constexpr (LONG && sizeof(T) == 4) {
+#pragma unroll
+          for (int ee = 0; ee < VEC; ++ee) acc[ee] += sum[ee];
         }
       } else {
 #pragma unroll 2
