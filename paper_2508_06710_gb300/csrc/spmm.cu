@@ -62,7 +62,7 @@ std::vector<int> vec_candidates(int eb, int k) {
 //   long rows (12 to 40 entries: the 13- and 27-point operators').  FP32: the TMA ring, whose entries
 //     come from shared memory while eight or more gathers per lane are in flight (27p k = 1, 3, 8
 //     137, 163, 216 and with the row split over lanes 185, 224, 353; 13p k = 1, 3 74, 86 and 91, 107;
-//     not 13p k = 8, 140 and direct 134; 27p k = 4 in halves, 164 against 168).  FP64 is
+//     13p k = 8 140 and direct 134, but its error is a quarter smaller in the ring; 27p k = 4 in halves, 164 against 168).  FP64 is
 //     bound by its pipe and splitting a row pays shuffles on it: one lane per row, in the ring where
 //     loads still matter (27p k = 1, 2, 3 239, 380, 570 and direct 291, 397, 662; 13p k = 1 109 and
 //     129), direct otherwise (13p k = 3 275, in the ring 292; with eight lanes per row, the choice
@@ -109,7 +109,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
     }
     if (op->format == RB_CSR && f64 && k >= 2 && len >= 4.0) t.grid_cap = 0;
     const double matrix = (double)op->nnz * (4 + eb) + 4.0 * op->n_rows;
-    const bool ring = mid ? (f32 ? k < 8 || len >= 20.0 : k == 1 || (len >= 20.0 && k <= 3))
+    const bool ring = mid ? (f32 ? k <= 8 || len >= 20.0 : k == 1 || (len >= 20.0 && k <= 3))
                           : csr && f32 && matrix > 100e6 && (len < 4.0 || (many && w == 4)) && op->n_rblk <= 1;
     if (ring && even) {
       SpmmSched r = t;

@@ -181,11 +181,11 @@ __global__ void __launch_bounds__(kTmaThreads, LONG ? (sizeof(T) == 4 ? 3 : 2) :
         int p = rs;
         T sum[LONG ? VEC : 1] = {};  // of an FP32 row's batches; the rest of the row sums in acc
         if constexpr (LONG) {
-          // FP32: a batch sums in four chains of its own, and its sum joins the row's, so rounding
-          // grows with the batches and not with the entries (27p k = 8, against 64 bits: 6.7e-8, as with
-          // the row split over lanes; one pair of chains through the row 8.3e-8 in 211 us).  FP64: one chain (a further addition
-          // takes a slot of its pipe).
-          constexpr int U = kLongGathers<T, VEC>, A = sizeof(T) == 4 ? 4 : 1;
+          // FP32: a batch sums in four or eight chains of its own, and its sum joins the row's, so
+          // rounding grows with the batches and not with the entries (27p k = 8, against 64 bits:
+          // 6.7e-8, as with the row split over lanes; one pair of chains through the row 8.3e-8 in
+          // 211 us).  FP64: one chain (a further addition takes a slot of its pipe).
+          constexpr int U = kLongGathers<T, VEC>, A = sizeof(T) == 4 ? (U == 13 ? 8 : 4) : 1;
           for (; p + U <= re; p += U) {
             Vec<T, VEC> x[U];
 #pragma unroll
@@ -200,10 +200,15 @@ __global__ void __launch_bounds__(kTmaThreads, LONG ? (sizeof(T) == 4 ? 3 : 2) :
                 else part[u % A][ee] = u < A ? v * x[u].v[ee] : fma(v, x[u].v[ee], part[u % A][ee]);
               }
             }
-            if constexpr (A == 4) {
+            if constexpr (A > 1) {
 #pragma unroll
-              for (int ee = 0; ee < VEC; ++ee)
-                sum[ee] += (part[0][ee] + part[1][ee]) + (part[2][ee] + part[3][ee]);
+              for (int h = A / 2; h >= 1; h /= 2)
+#pragma unroll
+                for (int q = 0; q < h; ++q)
+#pragma unroll
+                  for (int ee = 0; ee < VEC; ++ee) part[q][ee] += part[q + h][ee];
+#pragma unroll
+              for (int ee = 0; ee < VEC; ++ee) sum[ee] += part[0][ee];
             }
           }
         }
