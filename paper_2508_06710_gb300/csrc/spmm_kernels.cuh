@@ -86,6 +86,10 @@ rb_status launch_csr(const rb_op* op, const SpmmSched& sc, const T* X, int64_t l
   if (sc.stage == 2) {
     if constexpr (LPR == 1) {
       auto go = [&](auto* kern, int rows, int cap, size_t smem, int threads) -> rb_status {
+        if (rows < 4 || rows % 4) {  // the bulk copies of the row pointers start 16-byte aligned
+          set_error("spmm: the TMA pipeline takes tiles of a multiple of four rows, not %d", rows);
+          return RB_EUNSUPPORTED;
+        }
         RB_TRY(opt_in_smem(reinterpret_cast<const void*>(kern), smem));
         grid = wave_grid(kern, ((int64_t)op->n_rows + rows - 1) / rows, smem, threads);
         if (sc.grid_cap > 0) grid = std::min<int64_t>(grid, sc.grid_cap);  // fewer blocks, more tiles each

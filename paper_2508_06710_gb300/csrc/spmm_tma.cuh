@@ -33,10 +33,12 @@ template <typename T, int VEC>
 constexpr int kLongGathers = sizeof(T) * VEC >= 12 ? 8 : 13;
 constexpr int kTmaThreads = kThreads + 32;  // 8 consumer warps + 1 producer warp
 
-// consumer threads of a long-row block: 256, halved while its tile exceeds 32 KB
+// consumer threads of a long-row block: 256, halved while its tile exceeds 32 KB and half of them
+// would still hold a multiple of four rows (a tile's row pointers are one bulk copy, whose source
+// must be 16-byte aligned: every tile starts at a multiple of four rows)
 inline int tma_long_threads(double avg_row_len, int elem_bytes, int kp) {
   int c = kThreads;
-  while (c > 64 && c / 2 >= kp && (double)(c / kp) * avg_row_len * (4 + elem_bytes) > 32 * 1024) c /= 2;
+  while (c > 64 && c / 2 / kp % 4 == 0 && (double)(c / kp) * avg_row_len * (4 + elem_bytes) > 32 * 1024) c /= 2;
   return c;
 }
 
