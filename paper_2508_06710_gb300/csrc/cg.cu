@@ -1623,7 +1623,9 @@ struct UShared {
   double out[2 * K], tot[2 * K];
   double rz[K], alpha[K], beta[K];
   int state[K], iters[K], met[K];
-  int go, mine;
+  // go: another iteration; passed: unit_barrier's verdict, a word of its own, because a block whose
+  // system has finished reads it with no block barrier before the next iteration's go is written
+  int go, mine, passed;
 };
 
 // Block sums of the threads' per-float sums t[quantity][float]: column of float e is
@@ -1823,10 +1825,10 @@ __device__ bool unit_barrier(const PBatch& b, unsigned phase, UShared& sh) {
         }
       }
     }
-    sh.go = ok;
+    sh.passed = ok;
   }
   __syncthreads();
-  return sh.go != 0;
+  return sh.passed != 0;
 }
 
 // a block's partial of quantity q, batch column c: the blocks' values of one sum lie together
