@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "spmm_impl.cuh"
 
 namespace rb {
 
@@ -89,7 +90,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
   sc.stage = 0;
   sc.grid_cap = -1;
   std::vector<int> order;
-  if (mid && len >= 20.0 && (f64 ? k == 2 : k == 4)) order.push_back(k / 2);
+  if (mid && (f64 ? k == 2 && len >= 20.0 : k == 4 && len >= kEightSums)) order.push_back(k / 2);
   // (up to 32 columns: beyond, unaligned rows are refused, and four doubles need no alignment)
   if (csr && f64 && k % 4 == 0 && (k & (k - 1)) == 0 && k <= 32 && len < 12.0) order.push_back(4);
   if (many) order.push_back(4);

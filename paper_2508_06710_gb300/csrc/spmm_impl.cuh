@@ -157,6 +157,111 @@ __device__ __forceinline__ void extruded_epilogue(const CsrArgs<T>& a, int64_t r
   }
 }
 
+// A row that one lane walks sums in CH chains, entry q in chain q mod CH, which are added as a tree:
+// the order, and so the result bit for bit, of CH lanes that split the row (row_accumulate).  Rounding
+// grows with n ((n / CH + 1) / 2 + log2 CH) for n entries of like size, so eight chains pay from 16
+// entries on and four below (on the 13-point operator four are 1% better than eight).
+constexpr double kEightSums = 16.0;
+
+// The sum over a row's n entries, U (a multiple of CH) gathers in flight: gather(q) is entry q's piece of
+// X, value(q) its coefficient, read with the gather (EARLY: a global load) or at its use (shared memory).
+// The entries after the last full batch, FP32: whole groups of eight and four, the last three under
+// predicates (27-point k = 8, 150^3: 187 us, all seven under predicates 193).  FP64, whose predicated-off
+// FMAs still take slots of its pipe: a jump to the first that is there (k = 1: 246 us, predicates 260).
+template <typename T, int VEC, int CH, int U, bool EARLY, typename G, typename W>
+__device__ __forceinline__ void sum_in_chains(int n, G gather, W value, T (&acc)[VEC]) {
+  static_assert(U % CH == 0 && U <= 16, "whole turns of the chains");
+  T part[CH][VEC], v[U];
+  Vec<T, VEC> x[U];
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) part[c][e] = T(0);
+  int q = 0;  // the batch's first entry
+  auto get = [&](int u) {
+    if (u >= U) return;  // (unrolled indices of narrower batches)
+    if (EARLY) v[u] = value(q + u);
+    x[u] = gather(q + u);
+  };
+  auto add = [&](int u) {
+    if (u >= U) return;
+    const T w = EARLY ? v[u] : value(q + u);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) part[u % CH][e] = fma(w, x[u].v[e], part[u % CH][e]);
+  };
+  for (; q + U <= n; q += U) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) get(u);
+#pragma unroll
+    for (int u = 0; u < U; ++u) add(u);
+  }
+  const int m = n - q;
+  if constexpr (sizeof(T) == 4) {
+    auto last7 = [&](int o, int left) {
+      if (U > 4 && left >= 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) get(o + u);
+#pragma unroll
+        for (int u = 4; u < 7; ++u)
+          if (u < left) get(o + u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) add(o + u);
+#pragma unroll
+        for (int u = 4; u < 7; ++u)
+          if (u < left) add(o + u);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+          if (u < left) get(o + u);
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+          if (u < left) add(o + u);
+      }
+    };
+    if (U > 8 && m >= 8) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) get(u);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) add(u);
+      last7(8, m - 8);
+    } else {
+      last7(0, m);
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+      if (u < m) get(u);
+    auto last = [&](int o, int left) {  // left < CH: each in a chain of its own, in any order
+      switch (left) {
+        case 7: add(o + 6);
+        case 6: add(o + 5);
+        case 5: add(o + 4);
+        case 4: add(o + 3);
+        case 3: add(o + 2);
+        case 2: add(o + 1);
+        case 1: add(o);
+        default: break;
+      }
+    };
+    static_assert(sizeof(T) == 4 || U <= 2 * CH, "at most one full turn before the last entries");
+    if (U > CH && m >= CH) {
+#pragma unroll
+      for (int u = 0; u < CH; ++u) add(u);
+      last(CH, m - CH);
+    } else {
+      last(0, m);
+    }
+  }
+#pragma unroll
+  for (int h = CH / 2; h >= 1; h /= 2)
+#pragma unroll
+    for (int c = 0; c < h; ++c)
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) part[c][e] += part[c + h][e];
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) acc[e] = part[0][e];
+}
+
 // Direct accumulation for one (row, chunk, sub) without shared-memory staging: the row's
 // index and value loads are issued by all KP * LPR lanes of the row and served as one
 // broadcast.  Must be called by every lane of the warp when LPR > 1.

@@ -100,10 +100,18 @@ rb_status launch_csr(const rb_op* op, const SpmmSched& sc, const T* X, int64_t l
       if (op->avg_row_len >= 12.0) {
         const int consumers = tma_long_threads(op->avg_row_len, sizeof(T), sc.kp), rows = consumers / sc.kp;
         const int cap = tma_capacity<T, true>(op, rows, kTmaSmemLimit);
-        return go(&k_spmm_tma<T, VEC, EPI, true>, rows, cap, tma_layout<T, true>(rows, cap).total, consumers + 32);
+        const size_t smem = tma_layout<T, true>(rows, cap).total;
+        // the parts of a row's sum (spmm_tma.cuh)
+        if constexpr (sizeof(T) == 4 && VEC <= 2)
+          if (op->avg_row_len >= 13.0 && op->avg_row_len < kEightSums && (sc.kp == 1 || sc.kp >= 8))
+            return go(&k_spmm_tma<T, VEC, EPI, 13>, rows, cap, smem, consumers + 32);
+        if constexpr (VEC < 4)
+          if (k <= 4 && op->avg_row_len >= kEightSums)
+            return go(&k_spmm_tma<T, VEC, EPI, 8>, rows, cap, smem, consumers + 32);
+        return go(&k_spmm_tma<T, VEC, EPI, 4>, rows, cap, smem, consumers + 32);
       }
       const int cap = tma_capacity<T, false>(op, R, kTmaSmemLimit);
-      return go(&k_spmm_tma<T, VEC, EPI, false>, R, cap, tma_layout<T, false>(R, cap).total, kTmaThreads);
+      return go(&k_spmm_tma<T, VEC, EPI, 0>, R, cap, tma_layout<T, false>(R, cap).total, kTmaThreads);
     }
     set_error("spmm: the TMA pipeline takes one lane per row");
     return RB_EUNSUPPORTED;

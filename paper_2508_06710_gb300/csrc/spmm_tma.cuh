@@ -23,14 +23,17 @@ namespace rb {
 // Two shapes of the ring.  Short rows: three stages and a block's usual 256 consumer threads.  Long
 // rows (LONG): a tile is tens of KB, so two stages and as many consumers as keep a tile near 28 KB
 // (four blocks per SM), and each lane issues kLongGathers gathers before it uses the first: a row's
-// gathers are an L2 round trip each, and two at a time left the 16 resident consumer warps waiting.
-// 160^3 27-point operator, FP32 k = 8: 216 us (1.16 GB: 0.80 of the measured HBM rate; three blocks
-// per SM, left to itself the compiler fits two: 254); with three stages 347, two gathers at a time
-// over 380, direct with eight threads a row 353; 13-point, k = 4: 90 us against 105 (direct).
+// gathers are an L2 round trip each, and two at a time left the 16 resident consumer warps waiting.  A
+// row's sum has the parts that lanes would make of it (spmm_impl.cuh): eight, four above four columns
+// or with four columns a lane.  27-point operator, FP32 k = 8, 150^3: 187 us (957 MB: 0.76 of the measured
+// HBM rate), error against 64 bits 6.25e-8, as with the row split over four lanes (292 us); in two running
+// chains 8.3e-8.  FP64 k = 1: 246 us and 1.06e-16 (one chain 206 and 1.75e-16, eight lanes 482 and 1.06e-16).
+// Three stages, two gathers at a time or two blocks per SM all took longer (k = 8, 160^3: 347, over 380 and
+// 254 us where this shape took 216).
 template <bool LONG>
 constexpr int kTmaStages = LONG ? 2 : 3;
-template <typename T, int VEC>
-constexpr int kLongGathers = sizeof(T) * VEC >= 12 ? 8 : 13;
+template <typename T, int VEC, int CH>
+constexpr int kLongGathers = sizeof(T) == 4 && CH == 8 && VEC <= 2 ? 16 : 8;
 constexpr int kTmaThreads = kThreads + 32;  // 8 consumer warps + 1 producer warp
 
 // consumer threads of a long-row block: 256, halved while its tile exceeds 32 KB and half of them
@@ -78,8 +81,11 @@ inline int tma_capacity(const rb_op* op, int R, size_t limit) {
   return cap;
 }
 
-template <typename T, int VEC, int EPI, bool LONG>
-__global__ void __launch_bounds__(kTmaThreads, LONG ? (sizeof(T) == 4 ? 3 : 2) : 0) k_spmm_tma(CsrArgs<T> a, int R, int cap, int* __restrict__ err) {
+// CH: 0 the short-row shape, otherwise the long-row one with CH partial sums a row
+template <typename T, int VEC, int EPI, int CH>
+__global__ void __launch_bounds__(kTmaThreads, CH ? (sizeof(T) == 4 ? 3 : 2) : 0)
+    k_spmm_tma(CsrArgs<T> a, int R, int cap, int* __restrict__ err) {
+  constexpr bool LONG = CH > 0;
   extern __shared__ __align__(128) unsigned char sm[];
   constexpr int kStages = kTmaStages<LONG>;
   const int consumers = (int)blockDim.x - 32;
@@ -180,51 +186,52 @@ __global__ void __launch_bounds__(kTmaThreads, LONG ? (sizeof(T) == 4 ? 3 : 2) :
       const int re = s_rp[rloc + 1] - p0a;
       const T* Xc = a.X + chunk * VEC;
       if (staged) {
-        int p = rs;
-        T sum[LONG ? VEC : 1] = {};  // of an FP32 row's batches; the rest of the row sums in acc
-        if constexpr (LONG) {
-          // FP32: a batch sums in four or eight chains of its own, and its sum joins the row's, so
-          // rounding grows with the batches and not with the entries (27p k = 8, against 64 bits:
-          // 6.7e-8, as with the row split over lanes; one pair of chains through the row 8.3e-8 in
-          // 211 us).  FP64: one chain (a further addition takes a slot of its pipe).
-          constexpr int U = kLongGathers<T, VEC>, A = sizeof(T) == 4 ? (U == 13 ? 8 : 4) : 1;
-          for (; p + U <= re; p += U) {
-            Vec<T, VEC> x[U];
+        if constexpr (CH == 13) {
+          // FP32 rows of 13 and a little more, up to two columns a lane (and not so few chunks that lanes
+          // would make four parts, which are no worse): thirteen gathers in one batch, whose eight chains
+          // join as a tree; the chains of one product join by FMA, without its rounding (13-point k = 1: 78
+          // us and 4.74e-8 against 64 bits, four chains 77 and 5.17e-8, eight lanes 179 and 5.22e-8)
+          int p = rs;
+          T sum[VEC] = {};
+          for (; p + 13 <= re; p += 13) {
+            Vec<T, VEC> x[13];
 #pragma unroll
-            for (int u = 0; u < U; ++u) x[u] = ldv<T, VEC>(Xc + (int64_t)s_ci[p + u] * a.ldx);
-            T part[A][VEC];
+            for (int u = 0; u < 13; ++u) x[u] = ldv<T, VEC>(Xc + (int64_t)s_ci[p + u] * a.ldx);
+            T part[8][VEC];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
+            for (int u = 0; u < 13; ++u) {
               const T v = s_va[p + u];
 #pragma unroll
-              for (int ee = 0; ee < VEC; ++ee) {
-                if constexpr (A == 1) acc[ee] = fma(v, x[u].v[ee], acc[ee]);
-                else part[u % A][ee] = u < A ? v * x[u].v[ee] : fma(v, x[u].v[ee], part[u % A][ee]);
-              }
+              for (int ee = 0; ee < VEC; ++ee)
+                part[u % 8][ee] = u < 8 ? v * x[u].v[ee] : fma(v, x[u].v[ee], part[u % 8][ee]);
             }
-            if constexpr (A > 1) {
 #pragma unroll
-              for (int h = A / 2; h >= 1; h /= 2)
+            for (int h = 4; h >= 1; h /= 2)
 #pragma unroll
-                for (int q = 0; q < h; ++q)
+              for (int q = 0; q < h; ++q)
 #pragma unroll
-                  for (int ee = 0; ee < VEC; ++ee) part[q][ee] += part[q + h][ee];
+                for (int ee = 0; ee < VEC; ++ee) part[q][ee] += part[q + h][ee];
 #pragma unroll
-              for (int ee = 0; ee < VEC; ++ee) sum[ee] += part[0][ee];
-            }
+            for (int ee = 0; ee < VEC; ++ee) sum[ee] += part[0][ee];
           }
-        }
-#pragma unroll 2
-        for (; p < re; ++p) {
-          const int c = s_ci[p];
-          const T v = s_va[p];
-          const Vec<T, VEC> x = ldv<T, VEC>(Xc + (int64_t)c * a.ldx);
-#pragma unroll
-          for (int ee = 0; ee < VEC; ++ee) acc[ee] = fma(v, x.v[ee], acc[ee]);
-        }
-        if constexpr (LONG && sizeof(T) == 4) {
+          sum_in_chains<T, VEC, 4, 4, false>(
+              re - p, [&](int q) { return ldv<T, VEC>(Xc + (int64_t)s_ci[p + q] * a.ldx); },
+              [&](int q) { return s_va[p + q]; }, acc);
 #pragma unroll
           for (int ee = 0; ee < VEC; ++ee) acc[ee] += sum[ee];
+        } else if constexpr (LONG) {
+          sum_in_chains<T, VEC, CH, kLongGathers<T, VEC, CH>, false>(
+              re - rs, [&](int q) { return ldv<T, VEC>(Xc + (int64_t)s_ci[rs + q] * a.ldx); },
+              [&](int q) { return s_va[rs + q]; }, acc);
+        } else {
+#pragma unroll 2
+          for (int p = rs; p < re; ++p) {
+            const int c = s_ci[p];
+            const T v = s_va[p];
+            const Vec<T, VEC> x = ldv<T, VEC>(Xc + (int64_t)c * a.ldx);
+#pragma unroll
+            for (int ee = 0; ee < VEC; ++ee) acc[ee] = fma(v, x.v[ee], acc[ee]);
+          }
         }
       } else {
 #pragma unroll 2
