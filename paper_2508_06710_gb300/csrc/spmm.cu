@@ -58,20 +58,24 @@ std::vector<int> vec_candidates(int eb, int k) {
 
 // The schedule of a call that nobody tuned.  Width: 16-byte vectors with one thread per row, then
 // three columns, then the widest aligned vector.  The other choices by measurement (us; channel
-// 192 x 128 x 96 Laplacian L, gradient G and divergence, 160^3 13- and 27-point operators, the
-// extruded mesh):
-//   long rows (12 to 40 entries: the 13- and 27-point operators').  FP32: the TMA ring, whose entries
-//     come from shared memory while eight or more gathers per lane are in flight (27p k = 1, 3, 8
-//     137, 163, 216 and with the row split over lanes 185, 224, 353; 13p k = 1, 3 74, 86 and 91, 107;
-//     13p k = 8 140 and direct 134, but its error is a quarter smaller in the ring; 27p k = 4 in halves, 164 against 168).  FP64 is
-//     bound by its pipe and splitting a row pays shuffles on it: one lane per row, in the ring where
-//     loads still matter (27p k = 1, 2, 3 239, 380, 570 and direct 291, 397, 662; 13p k = 1 109 and
-//     129), direct otherwise (13p k = 3 275, in the ring 292; with eight lanes per row, the choice
-//     before, 1129).  Longer rows than these operators', and few rows (24^3: too few for one lane each
-//     to hide its gathers, 27p FP32 k = 3 3.4 and in the ring 5.2), keep up to eight lanes.
+// 192 x 128 x 96 Laplacian L, gradient G and divergence, 150^3 13- and 27-point operators 13p and 27p,
+// the extruded mesh):
+//   long rows (12 entries on).  A row's sum has up to eight parts, fewer with more columns: eight lanes
+//     split the row while each still has a few chunks.  Where the rows are of like length, 12 to 40
+//     entries and enough of them (rows_by_chains), the parts are chains of one lane: the same sums
+//     without the shuffles (eight lanes took 13p FP64 k = 1, 3 375 and 935, 27p 482 and 1236).  Rows of
+//     uneven length keep the lanes, and so do few rows (24^3: too few for one lane each to hide its
+//     gathers, 27p FP32 k = 3 3.4 and in the ring 5.2).
+//   the chains in the TMA ring.  FP32, whose loads matter most, always, but for rows below 20 entries with
+//     more columns than a row has parts (27p k = 1, 3, 8 131, 153, 187 and direct 195, 221, 287; 13p k = 1,
+//     3, 8, 12 76, 83, 119, 203 and direct 88, 107, 139, 214; 27p k = 4 in halves, eight parts, 156).  FP64 is
+//     bound by its pipe: the ring for one column and 27p k = 2 in halves (13p k = 1 113 and direct 135; 27p
+//     246 and 269, k = 2 414 and 437), direct otherwise (13p k = 2, 3 193, 281 and in the ring 199, 305; 27p
+//     k = 3, 4 619, 680 and 640, 831).
 //   grid, direct kernels.  FP64 with two columns or more: one block per row block, not a resident
-//     wave (L k = 3 91 and 97, k = 8 226 and 248, extruded k = 64 150 and 157); one column and the
-//     gradient's rows of two: the wave (G k = 3 86 and 93).  FP32: the wave.
+//     wave (L k = 3 91 and 97, k = 8 226 and 248, extruded k = 64 150 and 157; 27p k = 4 680 and 738); one
+//     column, the gradient's rows of two and eight chains: the wave (G k = 3 86 and 93; 27p k = 3 619 and
+//     641).  FP32 and rows split over lanes: the wave.
 //   width.  FP64 k = 4, 8, 16, 32 on short rows: four doubles a thread (G k = 4 107 and 115, the
 //     divergence k = 8 191 and 224 with the grid).
 //   the TMA ring on short rows.  FP32, a matrix that does not stay in L2, and little work per entry
@@ -83,7 +87,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
   const bool csr = op->format == RB_CSR && op->ext_nz == 0;
   const double len = op->avg_row_len;
   const bool even = op->max_row_len <= 1.25 * len + 1.0;  // every tile within the ring's capacity
-  const bool mid = csr && len >= 12.0 && len < 40.0 && (f64 || f32) && op->n_rows > 24000;
+  const bool mid = rows_by_chains(op);
   const bool many = csr && f32 && k >= 12 && k % 4 == 0 && len < 12.0;
   SpmmSched sc;
   sc.lpr = 1;
@@ -104,17 +108,19 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
     if (k % w) continue;
     t.kp = next_pow2(k / w);
     if (!sched_valid(op, t, k, ldx, ldy, X, Y)) continue;
-    if (!mid && op->format != RB_SELL && len >= 12.0) {
+    if (op->format != RB_SELL && len >= 12.0) {
       t.lpr = std::max(1, std::min(8, 32 / t.kp / 4));
+      if (mid && len < kEightSums) t.lpr = std::min(t.lpr, 4);
       if (!sched_valid(op, t, k, ldx, ldy, X, Y)) t.lpr = 1;
     }
-    if (op->format == RB_CSR && f64 && k >= 2 && len >= 4.0) t.grid_cap = 0;
+    if (op->format == RB_CSR && f64 && k >= 2 && len >= 4.0 && (mid ? t.lpr < 8 : t.lpr == 1)) t.grid_cap = 0;
     const double matrix = (double)op->nnz * (4 + eb) + 4.0 * op->n_rows;
-    const bool ring = mid ? (f32 ? k <= 8 || len >= 20.0 : k == 1 || (len >= 20.0 && k <= 3))
+    const bool ring = mid ? (f32 ? t.lpr > 1 || k <= 8 || len >= 20.0 : k == 1 || (len >= 20.0 && k == 2))
                           : csr && f32 && matrix > 100e6 && (len < 4.0 || (many && w == 4)) && op->n_rblk <= 1;
     if (ring && even) {
       SpmmSched r = t;
       r.stage = 2;
+      r.lpr = 1;
       r.grid_cap = 0;
       if (sched_valid(op, r, k, ldx, ldy, X, Y)) t = r;
     }

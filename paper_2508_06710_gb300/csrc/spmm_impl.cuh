@@ -157,6 +157,14 @@ __device__ __forceinline__ void extruded_epilogue(const CsrArgs<T>& a, int64_t r
   }
 }
 
+// Rows of 12 to 40 entries of like length (the 13- and 27-point operators' kind), enough of them for one
+// lane each to fill the chip: their sums' parts are chains of one lane rather than lanes.
+inline bool rows_by_chains(const rb_op* op) {
+  const double len = op->avg_row_len;
+  return op->format == RB_CSR && op->ext_nz == 0 && op->n_rblk <= 1 && (op->dtype == RB_F64 || op->dtype == RB_F32) &&
+         op->n_rows > 24000 && len >= 12.0 && len < 40.0 && op->max_row_len <= 1.25 * len + 1.0;
+}
+
 // A row that one lane walks sums in CH chains, entry q in chain q mod CH, which are added as a tree:
 // the order, and so the result bit for bit, of CH lanes that split the row (row_accumulate).  Rounding
 // grows with n ((n / CH + 1) / 2 + log2 CH) for n entries of like size, so eight chains pay from 16
@@ -306,6 +314,16 @@ __device__ __forceinline__ void row_accumulate_direct(const CsrArgs<T>& a, int64
   }
 }
 
+// The same sum by one lane per row, in CH chains: no shuffles, several gathers in flight.
+template <typename T, int VEC, int CH>
+__device__ __forceinline__ void row_accumulate_chains(const CsrArgs<T>& a, int64_t row, int chunk, T (&acc)[VEC]) {
+  const int rs = __ldg(a.rp + row), re = __ldg(a.rp + row + 1);
+  const T* Xc = a.X + chunk * VEC;
+  sum_in_chains<T, VEC, CH, CH, true>(
+      re - rs, [&](int q) { return ldv<T, VEC>(Xc + (int64_t)__ldg(a.ci + rs + q) * a.ldx); },
+      [&](int q) { return __ldg(a.va + rs + q); }, acc);
+}
+
 // Epilogue variants, chosen at compile time so that a launch without a column scale or
 // without the spanwise coupling issues none of their instructions (not even predicated off).
 constexpr int kEpiExt = 1;    // extruded operator: add the periodic spanwise second difference
@@ -368,6 +386,20 @@ __global__ void __launch_bounds__(kThreads) k_spmm_direct(CsrArgs<T> a) {
     for (int e = 0; e < VEC; ++e) acc[e] = T(0);
     row_accumulate_direct<T, VEC, LPR>(a, row, chunk, sub, active, acc);
     if (active && sub == 0) store_row<T, VEC, EPI>(a, row, chunk, acc);
+  }
+}
+
+// One lane per row and chunk whose sum has as many parts as lanes would make (row_accumulate_chains).
+template <typename T, int VEC, int CH, int EPI>
+__global__ void __launch_bounds__(kThreads) k_spmm_chains(CsrArgs<T> a) {
+  const int R = kThreads / a.kp;
+  const int chunk = threadIdx.x % a.kp;
+  const int rloc = threadIdx.x / a.kp;
+  if (chunk * VEC >= a.k) return;
+  for (int64_t row = (int64_t)blockIdx.x * R + rloc; row < a.n_rows; row += (int64_t)gridDim.x * R) {
+    T acc[VEC];
+    row_accumulate_chains<T, VEC, CH>(a, row, chunk, acc);
+    store_row<T, VEC, EPI>(a, row, chunk, acc);
   }
 }
 

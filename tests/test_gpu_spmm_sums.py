@@ -1,5 +1,6 @@
-"""Rounding of the SpMM's long rows: a row that one lane walks in the ring sums in as many parts as the
-lanes that would split it, so its result equals theirs bit for bit (GPU)."""
+"""Rounding of the SpMM's long rows: a row that one lane walks, in the ring or direct, sums in as many
+parts as the lanes that would split it, so its result equals theirs bit for bit; rows of uneven length
+and hinted row blocks are split over lanes (GPU)."""
 import numpy as np
 import pytest
 import torch
@@ -10,6 +11,9 @@ from tests.conftest import to_dev
 from tests.test_gpu_spmm_long_rows import _matrix
 
 pytestmark = pytest.mark.gpu
+
+N = 24500  # above the row count from which one lane takes a row
+FEW = 3000
 
 
 def _run(op, X, c=None):
@@ -62,3 +66,42 @@ def test_rows_of_13_lose_nothing(rb, k):
         ring = np.linalg.norm(_run(op, X) - ref)
         op.set_schedule(k, vec, _lanes(k, vec), 0, -1)
         assert ring <= np.linalg.norm(_run(op, X) - ref), vec
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("lens", [(12,), (13,), (15, 16), (27,), (36, 39)])
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 5, 6, 8, 9, 12, 16])
+def test_default_schedule_sums_as_lanes_do(rb, dtype, lens, k):
+    A = _matrix(N, lens, 21)
+    op = rb.Operator.from_scipy(A, dtype=dtype, k_max=k)
+    X = _x(N, k, dtype, 90 + k)
+    s = op.schedule(X, torch.empty_like(X))
+    few = rb.Operator.from_scipy(A[:FEW], dtype=dtype, k_max=k)
+    wide = few.schedule(X, torch.empty((FEW, k), dtype=X.dtype, device="cuda"))
+    long = np.mean(lens) >= 16
+    parts = s["lpr"] if s["stage"] == 0 else (8 if long and k <= 4 and s["vec"] < 4 else 4)
+    assert parts >= (wide["lpr"] if long else min(4, wide["lpr"])), (s, wide)
+    if s["stage"] == 2 and dtype == "f32" and s["vec"] <= 2 and 13 <= np.mean(lens) < 16:
+        return  # the batch of 13: test_rows_of_13_lose_nothing
+    got = _run(op, X)[:FEW]
+    while parts * (s_kp := 8 // _lanes(k, s["vec"])) > 32:
+        parts //= 2
+    few.set_schedule(k, s["vec"], parts, 0, -1)
+    assert np.array_equal(got, _run(few, X)), (s, parts)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 8, 9, 16])
+def test_uneven_rows_and_row_blocks_keep_the_lanes(rb, dtype, k):
+    A = _matrix(N, (12, 12, 12, 60), 31)  # average 24, maximum 60
+    op = rb.Operator.from_scipy(A, dtype=dtype, k_max=k)
+    few = rb.Operator.from_scipy(A[:FEW], dtype=dtype, k_max=k)
+    X = _x(N, k, dtype, 95 + k)
+    s = op.schedule(X, torch.empty_like(X))
+    assert s == few.schedule(X, torch.empty((FEW, k), dtype=X.dtype, device="cuda"))
+    assert (s["lpr"], s["stage"], s["grid_cap"]) == (_lanes(k, s["vec"]), 0, 0 if s["lpr"] == 1 and dtype == "f64" else -1)
+    assert np.array_equal(_run(op, X)[:FEW], _run(few, X))
+    even = rb.Operator.from_scipy(_matrix(N, (27,), 32), dtype=dtype, k_max=k)
+    even.set_row_blocks([0, 8000, 16000])
+    h = even.schedule(X, torch.empty_like(X))
+    assert (h["lpr"], h["stage"]) == (_lanes(k, h["vec"]), 0)
