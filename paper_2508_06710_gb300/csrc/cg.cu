@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -29,8 +30,7 @@
 
 namespace rb {
 
-SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X, const void* Y);
-SpmmSched pick_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X, const void* Y);
+SpmmSched solver_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X, const void* Y);
 
 namespace {
 
@@ -108,7 +108,23 @@ __device__ __forceinline__ void recount(CgScal* sc, int k) {
 
 // ------------------------------------------------------------------------- q = A p, p . q
 
-template <typename T, int VEC, int LPR>
+// A row of A times the thread's columns: LPR lanes split the row, or (CH > 1, LPR 1) one lane walks it in
+// CH chains, the same sum.  Poisson solves on 96^3, lanes and chains, ms: 13-point FP64 CG k = 1, 3, 8 54,
+// 129, 135 and 28, 58, 117, FP32-inner refinement 33, 53, 64 and 21, 29, 44; 27-point 40, 97, 127 and 27, 61,
+// 110, refinement 27, 41, 48 and 31, 32, 42 (one FP32 column: eight lanes' loads of a row's entries are one
+// piece, and stay; one chain a row, without the precision: 13-point 31, 54, 116 and 20, 31, 45).
+template <typename T, int VEC, int LPR, int CH, bool KEEP>
+__device__ __forceinline__ void row_product(const CsrArgs<T>& a, int64_t row, int chunk, int sub, bool active,
+                                            T (&acc)[VEC]) {
+  static_assert(CH == 1 || LPR == 1, "lanes or chains");
+  if constexpr (CH == 1) {
+    row_accumulate_direct<T, VEC, LPR, false, KEEP>(a, row, chunk, sub, active, acc);
+  } else {
+    if (active) row_accumulate_chains<T, VEC, CH, KEEP>(a, row, chunk, acc);
+  }
+}
+
+template <typename T, int VEC, int LPR, int CH>
 __global__ void __launch_bounds__(kThreads) k_cg_q(CsrArgs<T> a, CgCtl ctl, CgScal* __restrict__ sc,
                                                     double* __restrict__ partials) {
   if (sc->n_active == 0) return;
@@ -124,7 +140,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_q(CsrArgs<T> a, CgCtl ctl, CgSc
     T acc[VEC];
 #pragma unroll
     for (int e = 0; e < VEC; ++e) acc[e] = T(0);
-    row_accumulate_direct<T, VEC, LPR, false, true>(a, row, chunk, sub, active, acc);
+    row_product<T, VEC, LPR, CH, true>(a, row, chunk, sub, active, acc);
     if (active && sub == 0) {
       const Vec<T, VEC> p = ldv<T, VEC>(a.X + row * a.ldx + chunk * VEC);
       Vec<T, VEC> q;
@@ -307,7 +323,7 @@ __device__ __forceinline__ void q2_tail(DotAccN<T, 2 * VEC>& dacc, bool lead, in
   if (threadIdx.x == 0) recount(sc, k);
 }
 
-template <typename T, int VEC, int LPR>
+template <typename T, int VEC, int LPR, int CH>
 __global__ void __launch_bounds__(kThreads) k_cg_q2(CsrArgs<T> a, CgCtl ctl, const T* __restrict__ dinv,
                                                      CgScal* __restrict__ sc, double* __restrict__ partials) {
   if (sc->n_active == 0) return;
@@ -323,7 +339,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_q2(CsrArgs<T> a, CgCtl ctl, con
     T acc[VEC];
 #pragma unroll
     for (int e = 0; e < VEC; ++e) acc[e] = T(0);
-    row_accumulate_direct<T, VEC, LPR, false, true>(a, row, chunk, sub, active, acc);
+    row_product<T, VEC, LPR, CH, true>(a, row, chunk, sub, active, acc);
     if (active && sub == 0) {
       const Vec<T, VEC> p = ldv<T, VEC>(a.X + row * a.ldx + chunk * VEC);
       const T d = dinv ? dinv[row] : T(1);
@@ -487,7 +503,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_xrp(CgCtl ctl, T* __restrict__ 
 
 // ------------------------------------------------ true residual r = b - A x (FP64 operator)
 
-template <int VEC, int LPR>
+template <int VEC, int LPR, int CH>
 __global__ void __launch_bounds__(kThreads) k_cg_resid(CsrArgs<double> a, CgCtl ctl, int mode,
                                                         const double* __restrict__ B, int64_t ldb,
                                                         double* __restrict__ rout, CgScal* __restrict__ sc,
@@ -518,7 +534,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_resid(CsrArgs<double> a, CgCtl 
     double acc[VEC];
 #pragma unroll
     for (int e = 0; e < VEC; ++e) acc[e] = 0.0;
-    row_accumulate_direct<double, VEC, LPR>(a, row, chunk, sub, active, acc);
+    row_product<double, VEC, LPR, CH, false>(a, row, chunk, sub, active, acc);
     if (active && sub == 0) {
       const Vec<double, VEC> b = ldv<double, VEC>(B + row * ldb + chunk * VEC);
       Vec<double, VEC> rt;
@@ -905,27 +921,31 @@ struct Solver {
     return a;
   }
 
-  template <typename T, int VEC, int LPR>
-  void launch_q(const rb_op* op, const SpmmSched& ss, const T* p, T* q, CgCtl c) const {
-    CsrArgs<T> a = args<T>(op, ss, p, k, q, k);
-    k_cg_q<T, VEC, LPR><<<spmm_grid(&k_cg_q<T, VEC, LPR>, ss), kThreads, 0, s>>>(a, c, sc, partials);
+  // run(lanes per row, chains) as constants: the schedule's parts of a row's sum are lanes, or chains of
+  // one lane where the rows suit (the schedule then counts its blocks of rows with one lane each)
+  template <typename F>
+  static void by_parts(const rb_op* op, const SpmmSched& ss, F run) {
+    SpmmSched one = ss;
+    one.lpr = 1;
+    using I1 = std::integral_constant<int, 1>;
+    using I2 = std::integral_constant<int, 2>;
+    using I4 = std::integral_constant<int, 4>;
+    using I8 = std::integral_constant<int, 8>;
+    const bool chains = rows_by_chains(op) && !(op->dtype == RB_F32 && ss.lpr == 8 && ss.vec == 1);
+    switch (ss.lpr) {
+      case 2: chains ? run(one, I1(), I2()) : run(ss, I2(), I1()); break;
+      case 4: chains ? run(one, I1(), I4()) : run(ss, I4(), I1()); break;
+      case 8: chains ? run(one, I1(), I8()) : run(ss, I8(), I1()); break;
+      default: run(one, I1(), I1()); break;
+    }
   }
 
   template <typename T, int VEC>
   void launch_q_lpr(const rb_op* op, const SpmmSched& ss, const T* p, T* q, CgCtl c) const {
-    switch (ss.lpr) {
-      case 2: launch_q<T, VEC, 2>(op, ss, p, q, c); break;
-      case 4: launch_q<T, VEC, 4>(op, ss, p, q, c); break;
-      case 8: launch_q<T, VEC, 8>(op, ss, p, q, c); break;
-      default: launch_q<T, VEC, 1>(op, ss, p, q, c); break;
-    }
-  }
-
-  template <typename T, int VEC, int LPR>
-  void launch_q2(const rb_op* op, const SpmmSched& ss, const T* p, T* q, const T* dinv, CgCtl c) const {
-    CsrArgs<T> a = args<T>(op, ss, p, k, q, k);
-    k_cg_q2<T, VEC, LPR><<<spmm_grid(&k_cg_q2<T, VEC, LPR>, ss), kThreads, 0, s>>>(a, c, dinv, sc,
-                                                                                          partials);
+    by_parts(op, ss, [&](const SpmmSched& sd, auto lpr, auto ch) {
+      auto* kern = &k_cg_q<T, VEC, lpr.value, ch.value>;
+      kern<<<spmm_grid(kern, sd), kThreads, 0, s>>>(args<T>(op, sd, p, k, q, k), c, sc, partials);
+    });
   }
 
   template <typename T, int VEC>
@@ -960,29 +980,19 @@ struct Solver {
         return;
       }
     }
-    switch (ss.lpr) {
-      case 2: launch_q2<T, VEC, 2>(op, ss, p, q, dinv, c); break;
-      case 4: launch_q2<T, VEC, 4>(op, ss, p, q, dinv, c); break;
-      case 8: launch_q2<T, VEC, 8>(op, ss, p, q, dinv, c); break;
-      default: launch_q2<T, VEC, 1>(op, ss, p, q, dinv, c); break;
-    }
-  }
-
-  template <int VEC, int LPR>
-  void launch_resid_t(int mode, const double* B, int64_t ldb, const double* X, int64_t ldx, double* r) const {
-    CsrArgs<double> a = args<double>(A, sched64, X, ldx, nullptr, 0);
-    k_cg_resid<VEC, LPR><<<spmm_grid(&k_cg_resid<VEC, LPR>, sched64), kThreads, 0, s>>>(a, ctl, mode, B, ldb,
-                                                                                              r, sc, partials);
+    by_parts(op, ss, [&](const SpmmSched& sd, auto lpr, auto ch) {
+      auto* kern = &k_cg_q2<T, VEC, lpr.value, ch.value>;
+      kern<<<spmm_grid(kern, sd), kThreads, 0, s>>>(args<T>(op, sd, p, k, q, k), c, dinv, sc, partials);
+    });
   }
 
   template <int VEC>
   void launch_resid_v(int mode, const double* B, int64_t ldb, const double* X, int64_t ldx, double* r) const {
-    switch (sched64.lpr) {
-      case 2: launch_resid_t<VEC, 2>(mode, B, ldb, X, ldx, r); break;
-      case 4: launch_resid_t<VEC, 4>(mode, B, ldb, X, ldx, r); break;
-      case 8: launch_resid_t<VEC, 8>(mode, B, ldb, X, ldx, r); break;
-      default: launch_resid_t<VEC, 1>(mode, B, ldb, X, ldx, r); break;
-    }
+    by_parts(A, sched64, [&](const SpmmSched& sd, auto lpr, auto ch) {
+      auto* kern = &k_cg_resid<VEC, lpr.value, ch.value>;
+      kern<<<spmm_grid(kern, sd), kThreads, 0, s>>>(args<double>(A, sd, X, ldx, nullptr, 0), ctl, mode, B, ldb, r, sc,
+                                                    partials);
+    });
   }
 };
 
@@ -2130,12 +2140,12 @@ rb_status init_solver(Solver& S_, rb_op_t A, rb_op_t A_inner, const rb_cg_params
   S_.vec = vec;
   S_.kp = next_pow2(k / vec);
   RB_REQUIRE(S_.kp <= 32, "solve: k = %d needs 16-byte aligned B and X rows", k);
-  S_.sched64 = pick_sched(A, k, k, k, base + L.r, base + L.p);
+  S_.sched64 = solver_sched(A, k, k, k, base + L.r, base + L.p);
   S_.sched64.vec = vec;
   S_.sched64.kp = S_.kp;
   if (S_.sched64.kp * S_.sched64.lpr > 32) S_.sched64.lpr = 1;
   if (prm.mixed) {
-    S_.sched32 = pick_sched(A_inner, k, k, k, base + L.p32, base + L.q32);
+    S_.sched32 = solver_sched(A_inner, k, k, k, base + L.p32, base + L.q32);
     S_.sched32.vec = vec;  // the same (row, chunk) layout as the vector kernels
     S_.sched32.kp = S_.kp;
     if (S_.sched32.kp * S_.sched32.lpr > 32) S_.sched32.lpr = 1;

@@ -81,7 +81,9 @@ std::vector<int> vec_candidates(int eb, int k) {
 //   the TMA ring on short rows.  FP32, a matrix that does not stay in L2, and little work per entry
 //     loaded (rows of two: G k = 3 49 and 58) or many columns (L k = 16 88 and 99).
 // The ring is taken only where every tile fits its stages (no row far above the average).
-SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X, const void* Y) {
+// (`pipelined` false: a caller with kernels of its own, whose rows are read directly.)
+SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X, const void* Y,
+                        bool pipelined = true) {
   const int eb = op->dtype == RB_F32 ? 4 : 8;
   const bool f64 = op->dtype == RB_F64, f32 = op->dtype == RB_F32;
   const bool csr = op->format == RB_CSR && op->ext_nz == 0;
@@ -94,7 +96,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
   sc.stage = 0;
   sc.grid_cap = -1;
   std::vector<int> order;
-  if (mid && (f64 ? k == 2 && len >= 20.0 : k == 4 && len >= kEightSums)) order.push_back(k / 2);
+  if (mid && pipelined && (f64 ? k == 2 && len >= 20.0 : k == 4 && len >= kEightSums)) order.push_back(k / 2);
   // (up to 32 columns: beyond, unaligned rows are refused, and four doubles need no alignment)
   if (csr && f64 && k % 4 == 0 && (k & (k - 1)) == 0 && k <= 32 && len < 12.0) order.push_back(4);
   if (many) order.push_back(4);
@@ -117,7 +119,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
     const double matrix = (double)op->nnz * (4 + eb) + 4.0 * op->n_rows;
     const bool ring = mid ? (f32 ? t.lpr > 1 || k <= 8 || len >= 20.0 : k == 1 || (len >= 20.0 && k == 2))
                           : csr && f32 && matrix > 100e6 && (len < 4.0 || (many && w == 4)) && op->n_rblk <= 1;
-    if (ring && even) {
+    if (ring && even && pipelined) {
       SpmmSched r = t;
       r.stage = 2;
       r.lpr = 1;
@@ -166,6 +168,13 @@ SpmmSched pick_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const voi
   auto it = op->tuned.find(k);
   if (it != op->tuned.end() && sched_valid(op, it->second, k, ldx, ldy, X, Y)) return it->second;
   return default_sched(op, k, ldx, ldy, X, Y);
+}
+
+// The schedule whose lanes per row the solvers' own products take (they read rows directly).
+SpmmSched solver_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X, const void* Y) {
+  auto it = op->tuned.find(k);
+  if (it != op->tuned.end() && sched_valid(op, it->second, k, ldx, ldy, X, Y)) return it->second;
+  return default_sched(op, k, ldx, ldy, X, Y, false);
 }
 
 std::vector<SpmmSched> tune_candidates(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X,

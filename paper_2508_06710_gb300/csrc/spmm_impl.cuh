@@ -314,13 +314,20 @@ __device__ __forceinline__ void row_accumulate_direct(const CsrArgs<T>& a, int64
   }
 }
 
-// The same sum by one lane per row, in CH chains: no shuffles, several gathers in flight.
-template <typename T, int VEC, int CH>
+// The same sum by one lane per row, in CH chains: no shuffles, several gathers in flight (KEEP: see above).
+template <typename T, int VEC, int CH, bool KEEP = false>
 __device__ __forceinline__ void row_accumulate_chains(const CsrArgs<T>& a, int64_t row, int chunk, T (&acc)[VEC]) {
   const int rs = __ldg(a.rp + row), re = __ldg(a.rp + row + 1);
   const T* Xc = a.X + chunk * VEC;
+  uint64_t keep = 0;
+  if constexpr (KEEP) keep = l2_keep_policy();
   sum_in_chains<T, VEC, CH, CH, true>(
-      re - rs, [&](int q) { return ldv<T, VEC>(Xc + (int64_t)__ldg(a.ci + rs + q) * a.ldx); },
+      re - rs,
+      [&](int q) {
+        const T* x = Xc + (int64_t)__ldg(a.ci + rs + q) * a.ldx;
+        if constexpr (KEEP) return ldv_keep<T, VEC>(x, keep);
+        else return ldv<T, VEC>(x);
+      },
       [&](int q) { return __ldg(a.va + rs + q); }, acc);
 }
 
