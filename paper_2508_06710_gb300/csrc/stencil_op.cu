@@ -65,12 +65,15 @@ __global__ void __launch_bounds__(kThreads) k_spmm_stencil7_run(Stencil7<T> st, 
 // tabulated when the operator is made, with its scale:
 //   line: a = s w_y w_z, b_ym, b_yp = s w_z / d_y, b_zm, b_zp = s w_y / d_z, S = -(b_ym + ... + b_zp)
 //   cell: 1 / d_x below and above, their negated sum D, w_x
-// One or two columns per thread: y = a (x_- / d + x_+ / d + D x_0) + w_x (b . x_yz + S x_0), ten
-// operations a value and none per cell.  More columns: the seven entries formed first (8 operations
-// a cell: two products with a, four with w_x, and the diagonal's two), then seven a value.  Forming
-// entries and diagonal from the axis tables took 14 a cell and 8 a value.  190 x 127 x 95 (one cell
-// per thread before), k = 3: 162 -> 121 us (the pipe alone: 106); 192 x 128 x 96 (runs of four cells
-// before), k = 1, 2, 3, 4, 8: 97, 131, 169, 250, 490 -> 45, 86, 123, 168, 332 us.
+// y = a (x_- / d + x_+ / d + D x_0) + w_x (b . x_yz + S x_0): ten operations a value and none per cell;
+// forming entries and diagonal from the axis tables took 14 a cell and 8 a value.  Each bracket cancels by
+// itself, so its rounding stays small: against extended precision 0.7 to 1.25e-16 (2-norm, random values)
+// and 0.45 to 0.7e-16 of |A| |x| (smooth ones), rows of seven entries 1.3 to 1.6e-16 and 0.85 to 1.0e-16.
+// (Three columns and more with the seven entries formed from the tables, 8 operations a cell and 7 a value,
+// took 121 us at k = 3, with up to 3% more error than before; with four entries and the diagonal, 28
+// operations at k = 3, 117 us, and no gain on smooth values.)  190 x 127 x 95 (one cell per thread before),
+// k = 3: 162 -> 124 us (the pipe alone: 110); 192 x 128 x 96 (runs of four cells before), k = 1, 2, 3, 4, 8: 97,
+// 131, 169, 250, 490 -> 46, 86, 127, 168, 332 us.
 struct alignas(16) LineCoef {
   double a, bym, byp, bzm, bzp, s;
 };
@@ -108,30 +111,15 @@ __global__ void __launch_bounds__(kThreads) k_spmm_stencil7_f64(Stencil7<double>
     const CellCoef t = cells[i];
     const LineCoef l = lines[line];
     Vec<double, VEC> y;
-    if constexpr (VEC <= 2) {
 #pragma unroll
-      for (int q = 0; q < VEC; ++q) {
-        const double u = fma(t.d, x0.v[q], fma(t.p, xp.v[q], t.m * xm.v[q]));
-        double v = l.s * x0.v[q];
-        v = fma(l.bym, ym.v[q], v);
-        v = fma(l.byp, yp.v[q], v);
-        v = fma(l.bzm, um.v[q], v);
-        v = fma(l.bzp, up.v[q], v);
-        y.v[q] = fma(l.a, u, t.w * v);
-      }
-    } else {
-      const double cxm = l.a * t.m, cxp = l.a * t.p, cym = t.w * l.bym, cyp = t.w * l.byp, czm = t.w * l.bzm,
-                   czp = t.w * l.bzp, diag = fma(t.w, l.s, l.a * t.d);
-#pragma unroll
-      for (int q = 0; q < VEC; ++q) {
-        double v = diag * x0.v[q];
-        v = fma(cxm, xm.v[q], v);
-        v = fma(cxp, xp.v[q], v);
-        v = fma(cym, ym.v[q], v);
-        v = fma(cyp, yp.v[q], v);
-        v = fma(czm, um.v[q], v);
-        y.v[q] = fma(czp, up.v[q], v);
-      }
+    for (int q = 0; q < VEC; ++q) {
+      const double u = fma(t.d, x0.v[q], fma(t.p, xp.v[q], t.m * xm.v[q]));
+      double v = l.s * x0.v[q];
+      v = fma(l.bym, ym.v[q], v);
+      v = fma(l.byp, yp.v[q], v);
+      v = fma(l.bzm, um.v[q], v);
+      v = fma(l.bzp, up.v[q], v);
+      y.v[q] = fma(l.a, u, t.w * v);
     }
     if constexpr (SCALE) {
 #pragma unroll
@@ -152,7 +140,15 @@ __global__ void k_stencil7_lines(Stencil7<double> st, LineCoef* __restrict__ lin
       l.a = wy * st.w[2][z];
       l.bym = wz * st.ic[1][j], l.byp = wz * st.ic[1][j + 1];
       l.bzm = wy * st.ic[2][z], l.bzp = wy * st.ic[2][z + 1];
-      l.s = -((l.bym + l.byp) + (l.bzm + l.bzp));
+      // minus the sum of the four, rounded once (exact sums of two by Knuth's two-sum)
+      auto two_sum = [](double x, double y, double& err) {
+        const double z = x + y, t = z - x;
+        err = (x - (z - t)) + (y - t);
+        return z;
+      };
+      double e1, e2, e3;
+      const double sy = two_sum(l.bym, l.byp, e1), sz = two_sum(l.bzm, l.bzp, e2), st4 = two_sum(sy, sz, e3);
+      l.s = -(st4 + (e1 + e2 + e3));
       lines[t] = l;
     } else {
       const int i = t - n_lines;
