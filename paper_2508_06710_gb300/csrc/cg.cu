@@ -1334,7 +1334,7 @@ __device__ __forceinline__ void pblock_reduce(float (&acc)[NQ][VEC], int kp, int
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) warp_fold<float, VEC>(acc[q], kp);
-  if (lane < kp) {
+  if (lane < kp && lane * VEC < k) {  // (chunks beyond k: see RedSmem)
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
 #pragma unroll

@@ -14,7 +14,8 @@ namespace rb {
 
 constexpr int kWarps = kThreads / 32;
 
-// Shared scratch for block_reduce: kWarps * NQ * KP * VEC doubles (KP * VEC <= 64).
+// Shared scratch for block_reduce: 64 columns per warp and quantity.  KP is rounded up to a power of two,
+// so KP * VEC may exceed them (17 chunks of three columns: 96): chunks beyond k write nothing.
 template <int NQ>
 struct RedSmem {
   double v[kWarps][NQ][64];
@@ -34,8 +35,8 @@ __device__ __forceinline__ double block_reduce(A (&acc)[NQ][VEC], int kp, int lp
   const int width = kp * lpr;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) warp_fold<A, VEC>(acc[q], width);
-  if (lane < width && (lane % lpr) == 0) {
-    const int chunk = lane / lpr;
+  const int chunk = lane / lpr;
+  if (lane < width && (lane % lpr) == 0 && chunk * VEC < k) {
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
 #pragma unroll
