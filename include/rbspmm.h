@@ -498,7 +498,8 @@ rb_status rb_mg_vcycle(rb_mg_t mg, int32_t level, rb_dtype dtype, const double* 
 /* Solves A x_j = b_j for k <= k_max columns by PCG (Saad, Alg. 9.1) preconditioned by one
  * V-cycle per iteration.  params: rtol (true relative residual ||b - A x|| / ||b||, the mean
  * removed from both when project_mean), max_iter, check_every (iterations between host
- * reads of the per-column state), project_mean, and
+ * reads of the per-column state; a recorded refinement sweep ends by itself and is read once),
+ * project_mean, and
  *   mixed = 0: FP64 CG and cycle; the true residual is checked every check_every iterations
  *              (columns stop at the first check that meets rtol);
  *   mixed != 0: FP64 iterative refinement around the same PCG run in FP32 (operators,
@@ -507,8 +508,8 @@ rb_status rb_mg_vcycle(rb_mg_t mg, int32_t level, rb_dtype dtype, const double* 
  *              when that is looser) and updates x += ||r|| d in FP64; at most max_sweeps.
  * precond and persistent are ignored.  B (ldb), X (ldx; in: initial guess, out: solution,
  * zero-mean with project_mean): float64 DEVICE.  Synchronises `stream`; allocates nothing
- * (the hierarchy holds the vectors and CUDA graphs of the iterations, recorded on first use
- * for each k).  Returns the worst column status; report (may be NULL) as for rb_cg_solve
+ * (the hierarchy holds the vectors and the CUDA graphs, of the iterations or of a whole sweep,
+ * recorded on their second use for each k and kept for the last 32 shapes).  Returns the worst column status; report (may be NULL) as for rb_cg_solve
  * (iters: CG iterations, over all sweeps when mixed; spmm_calls: FP64 residuals). */
 rb_status rb_mg_solve(rb_mg_t mg, const rb_cg_params* params, const double* B, int64_t ldb, double* X, int64_t ldx,
                       int32_t k, rb_cg_report* report, rb_stream_t stream);

@@ -64,6 +64,7 @@ struct MgScal {
   int state[K], iters[K];
   // the true residual b - A x (FP64)
   double bb[K], tol2[K], mean[K], scale[K], rr_true[K];
+  double inner_rtol;  // a refinement sweep's target (the recorded sweeps read it here)
   int ostate[K];
   int n_active, n_oactive;
   int left;  // iterations a refinement solve may still run (max_iter at its start)
@@ -833,6 +834,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kThreads) k_mg_true_resid(CsrArgs<double> a, const double* __restrict__ b,
                                                              int64_t ldb, double* __restrict__ rt, int kind,
                                                              int project, double rtol2, int max_iter,
+                                                             double inner_rtol,
                                                              MgScal* __restrict__ sc,
                                                              double* __restrict__ partials) {
   __shared__ RedSmem<4> red;
@@ -904,7 +906,7 @@ __global__ void __launch_bounds__(kThreads) k_mg_true_resid(CsrArgs<double> a, c
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (kind == TR_INIT) sc->left = max_iter;
+    if (kind == TR_INIT) sc->left = max_iter, sc->inner_rtol = inner_rtol;
     mg_recount(sc, a.k);
   }
 }
@@ -915,8 +917,7 @@ __global__ void __launch_bounds__(kThreads) k_mg_true_resid(CsrArgs<double> a, c
 // with the sweep's inner target set per column and its state reopened.
 template <typename T, int VEC, int MODE>
 __global__ void __launch_bounds__(kThreads) k_mg_rhs(int64_t n, int k, int kp, const double* __restrict__ rt,
-                                                      T* __restrict__ out, MgScal* __restrict__ sc, double inner_rtol,
-                                                      double rtol) {
+                                                      T* __restrict__ out, MgScal* __restrict__ sc) {
   const int R = kThreads / kp;
   const int chunk = threadIdx.x % kp;
   if (chunk * VEC >= k) return;
@@ -941,7 +942,7 @@ __global__ void __launch_bounds__(kThreads) k_mg_rhs(int64_t n, int k, int kp, c
         // this sweep's target: inner_rtol of its residual, or only what the outer tolerance
         // still needs (half of it) when that is looser, so the last sweep does not overshoot
         const double need = 0.5 * sqrt(sc->tol2[j]) / sc->scale[j];
-        const double tgt = fmax(inner_rtol, need);
+        const double tgt = fmax(sc->inner_rtol, need);
         sc->itol2[j] = tgt * tgt;
         sc->state[j] = MG_ACTIVE;
       } else if (sc->state[j] == MG_ACTIVE) {
@@ -1120,15 +1121,21 @@ struct rb_mg {
   rb::MgScal* sc = nullptr;
   double* partials = nullptr;
   int64_t device_bytes = 0;
-  // CUDA graphs of check_every CG iterations, per (precision, k, chunk, flexible)
-  std::map<std::vector<int>, cudaGraphExec_t> graphs;
+  // CUDA graphs, of a refinement sweep per (-1, k, flexible) and of the FP64 CG's iterations per (8, k,
+  // their number, flexible); a null one marks a sweep that ran once, eagerly
+  struct Recorded {
+    cudaGraphExec_t exec = nullptr;
+    uint64_t used = 0;  // the hierarchy's launch count at its last use
+  };
+  std::map<std::vector<int>, Recorded> graphs;
+  uint64_t launches = 0;
   cudaStream_t cap = nullptr;  // private stream for graph capture
 };
 
 namespace rb {
 namespace {
 
-constexpr size_t kMgGraphs = 32;  // recorded shapes a hierarchy keeps
+constexpr size_t kMgGraphs = 32;  // shapes whose graphs a hierarchy keeps
 constexpr int kMgPartials = 4 * K * kMaxGrid;  // 4 quantities x k columns x blocks
 
 template <typename T>
@@ -1164,7 +1171,7 @@ void mg_free(rb_mg* g) {
                   (void*)g->partials})
     if (p) cudaFree(p);
   for (auto& kv : g->graphs)
-    if (kv.second) cudaGraphExecDestroy(kv.second);
+    if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
   if (g->cap) cudaStreamDestroy(g->cap);
   delete g;
 }
@@ -1635,48 +1642,67 @@ rb_status mg_read(rb_mg* g, MgHost& h, cudaStream_t s) {
   return RB_OK;
 }
 
+// The place of a shape's graph: of kMgGraphs shapes the one not used for longest goes (and is recorded
+// again should it return)
+rb_status graph_slot(rb_mg* g, const std::vector<int>& key, cudaStream_t s, rb_mg::Recorded** slot) {
+  if (g->graphs.size() >= kMgGraphs && !g->graphs.count(key)) {
+    auto old = g->graphs.begin();
+    for (auto it = old; it != g->graphs.end(); ++it)
+      if (it->second.used < old->second.used) old = it;
+    if (old->second.exec) {
+      RB_CUDA(cudaStreamSynchronize(s));
+      cudaGraphExecDestroy(old->second.exec);
+    }
+    g->graphs.erase(old);
+  }
+  *slot = &g->graphs[key];
+  (*slot)->used = ++g->launches;
+  return RB_OK;
+}
+
 // `chunk` CG iterations, recorded once per shape as a CUDA graph and replayed
 template <typename T, int VEC>
-rb_status run_iterations(rb_mg* g, const Cycle<T, VEC>& cy, bool inner, int flexible, int chunk, int& uses) {
-  const std::vector<int> key = {(int)sizeof(T), cy.k, chunk, flexible, inner ? 1 : 0};
-  auto it = g->graphs.find(key);
-  if (it == g->graphs.end() && uses == 0) {  // the first chunk runs eagerly (launch caches fill)
-    for (int i = 0; i < chunk; ++i) RB_TRY((cg_iteration<T, VEC>(g, cy, inner, flexible)));
+rb_status run_iterations(rb_mg* g, const Cycle<T, VEC>& cy, int flexible, int chunk, int& uses) {
+  const std::vector<int> key = {(int)sizeof(T), cy.k, chunk, flexible};
+  if (uses == 0 && !g->graphs.count(key)) {  // the first chunk runs eagerly (launch caches fill)
+    for (int i = 0; i < chunk; ++i) RB_TRY((cg_iteration<T, VEC>(g, cy, false, flexible)));
     ++uses;
     return RB_OK;
   }
-  if (it == g->graphs.end()) {
+  rb_mg::Recorded* rec = nullptr;
+  RB_TRY(graph_slot(g, key, cy.s, &rec));
+  if (!rec->exec) {
     if (!g->cap) RB_CUDA(cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking));
     Cycle<T, VEC> cc = cy;
     cc.s = g->cap;
     cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
     RB_CUDA(cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal));
     rb_status st = RB_OK;
-    for (int i = 0; i < chunk && st == RB_OK; ++i) st = cg_iteration<T, VEC>(g, cc, inner, flexible);
+    for (int i = 0; i < chunk && st == RB_OK; ++i) st = cg_iteration<T, VEC>(g, cc, false, flexible);
     cudaError_t e = cudaStreamEndCapture(g->cap, &graph);
     if (st != RB_OK) {
       if (graph) cudaGraphDestroy(graph);
       return st;
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&rec->exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
-    if (e != cudaSuccess) return cuda_fail(e, "CUDA graph of the multigrid CG iterations", __FILE__, __LINE__);
-    it = g->graphs.emplace(key, exec).first;
+    if (e != cudaSuccess) {
+      rec->exec = nullptr;
+      return cuda_fail(e, "CUDA graph of the multigrid CG iterations", __FILE__, __LINE__);
+    }
   }
-  RB_CUDA(cudaGraphLaunch(it->second, cy.s));
+  RB_CUDA(cudaGraphLaunch(rec->exec, cy.s));
   ++uses;
   return RB_OK;
 }
 
 // A refinement sweep's scaled FP32 residual, zero d, and the first z and p
 template <int VEC32>
-rb_status sweep_start(const rb_mg* g, const Cycle<float, VEC32>& cy, const rb_cg_params& prm) {
+rb_status sweep_start(const rb_mg* g, const Cycle<float, VEC32>& cy) {
   const int64_t n = g->lv[0].cells;
   RB_CUDA(cudaMemsetAsync(g->x, 0, sizeof(float) * (size_t)n * cy.k, cy.s));
   auto* kr = &k_mg_rhs<float, VEC32, 1>;
-  kr<<<cy.grid(kr, n), kThreads, 0, cy.s>>>(n, cy.k, cy.kp, g->rt, static_cast<float*>(g->r), g->sc, prm.inner_rtol,
-                                           prm.rtol);
+  kr<<<cy.grid(kr, n), kThreads, 0, cy.s>>>(n, cy.k, cy.kp, g->rt, static_cast<float*>(g->r), g->sc);
   return cg_start<float, VEC32>(g, cy);
 }
 
@@ -1698,8 +1724,7 @@ rb_status sweep_end(const rb_mg* g, const Cycle<float, VEC32>& cy) {
 // 7.70 -> 7.21 ms; projection step on 128^3, m = 2: 22.9 -> 21.0 ms.  exec stays null where the runtime cannot
 // record a loop node (the caller then goes on eagerly).
 template <int VEC32>
-rb_status sweep_graph(rb_mg* g, const Cycle<float, VEC32>& cy, const rb_cg_params& prm, int flexible,
-                      cudaGraphExec_t* exec) {
+rb_status sweep_graph(rb_mg* g, const Cycle<float, VEC32>& cy, int flexible, cudaGraphExec_t* exec) {
   *exec = nullptr;
   if (!g->cap) RB_CUDA(cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking));
   Cycle<float, VEC32> cc = cy;
@@ -1712,7 +1737,7 @@ rb_status sweep_graph(rb_mg* g, const Cycle<float, VEC32>& cy, const rb_cg_param
   cudaError_t e = cudaGraphConditionalHandleCreate(&loop, graph, 0, cudaGraphCondAssignDefault);
   if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(g->cap, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
-    st = sweep_start<VEC32>(g, cc, prm);
+    st = sweep_start<VEC32>(g, cc);
     if (st == RB_OK) st = cg_step<float, VEC32>(g, cc, true, loop);
     cudaStreamCaptureStatus cs;
     cudaGraph_t into = nullptr;
@@ -1758,7 +1783,7 @@ rb_status true_resid(rb_mg* g, const double* B, int64_t ldb, const double* X, do
   const int64_t n = g->lv[0].cells;
   const int grid = wave_grid(kern, (n + kThreads / kp - 1) / (kThreads / kp));
   kern<<<grid, kThreads, 0, s>>>(csr_args<double>(A, X, nullptr, k, kp), B, ldb, out, kind, prm.project_mean,
-                                 prm.rtol * prm.rtol, prm.max_iter, g->sc, g->partials);
+                                 prm.rtol * prm.rtol, prm.max_iter, prm.inner_rtol, g->sc, g->partials);
   RB_CUDA(cudaGetLastError());
   return RB_OK;
 }
@@ -1781,7 +1806,7 @@ rb_status mg_solve_vec(rb_mg* g, const rb_cg_params& prm, const double* B, int64
     RB_TRY(true_resid<VEC64>(g, B, ldb, x, g->rt, TR_INIT, k, kp64, prm, s));
     ++spmm64;
     auto* kr = &k_mg_rhs<double, VEC64, 0>;
-    kr<<<cy.grid(kr, n), kThreads, 0, s>>>(n, k, kp64, g->rt, static_cast<double*>(g->r), g->sc, 0.0, prm.rtol);
+    kr<<<cy.grid(kr, n), kThreads, 0, s>>>(n, k, kp64, g->rt, static_cast<double*>(g->r), g->sc);
     RB_TRY((cg_start<double, VEC64>(g, cy)));
     int it = 0;
     for (;;) {
@@ -1793,7 +1818,7 @@ rb_status mg_solve_vec(rb_mg* g, const rb_cg_params& prm, const double* B, int64
         break;
       }
       const int chunk = std::min(check, prm.max_iter - it);
-      RB_TRY((run_iterations<double, VEC64>(g, cy, false, flexible, chunk, uses)));
+      RB_TRY((run_iterations<double, VEC64>(g, cy, flexible, chunk, uses)));
       it += chunk;
       RB_TRY(true_resid<VEC64>(g, B, ldb, x, g->rt, TR_CHECK, k, kp64, prm, s));
       ++spmm64;
@@ -1807,11 +1832,9 @@ rb_status mg_solve_vec(rb_mg* g, const rb_cg_params& prm, const double* B, int64
     Cycle<float, VEC32> cy{g, k, kp32, s, &g->sc->n_active};
     double* x64 = g->x64;
     k_mg_copy<double, double><<<cg, 256, 0, s>>>(n, k, X, ldx, x64, k);
-    // the sweep's graph, kept per shape and inner tolerance; the hierarchy's first sweep of a shape
-    // runs eagerly, so that the launch-shape caches are filled before the recording
-    uint64_t tol_bits;
-    std::memcpy(&tol_bits, &prm.inner_rtol, 8);
-    const std::vector<int> key = {-1, k, flexible, (int)(uint32_t)tol_bits, (int)(uint32_t)(tol_bits >> 32)};
+    // the sweep's graph, one per k (the tolerances and max_iter lie on the device); a hierarchy's first
+    // sweep of a k runs eagerly, so that the launch-shape caches are filled before the recording
+    const std::vector<int> key = {-1, k, flexible};
     for (;; ++sweeps) {
       RB_TRY(true_resid<VEC64>(g, B, ldb, x64, g->rt, sweeps == 0 ? TR_INIT : TR_CHECK, k, kp64, prm, s));
       ++spmm64;
@@ -1822,26 +1845,15 @@ rb_status mg_solve_vec(rb_mg* g, const rb_cg_params& prm, const double* B, int64
         k_mg_mark_noconv<<<1, K, 0, s>>>(g->sc, k);
         break;
       }
-      auto it = g->graphs.find(key);
-      if (it != g->graphs.end() && !it->second) {
-        if (g->graphs.size() > kMgGraphs)  // other shapes and tolerances: recorded again when they return
-          for (auto o = g->graphs.begin(); o != g->graphs.end();) {
-            if (o == it || !o->second) {
-              ++o;
-            } else {
-              RB_CUDA(cudaStreamSynchronize(s));
-              cudaGraphExecDestroy(o->second);
-              o = g->graphs.erase(o);
-            }
-          }
-        RB_TRY(sweep_graph<VEC32>(g, cy, prm, flexible, &it->second));
-      }
-      if (it != g->graphs.end() && it->second) {
-        RB_CUDA(cudaGraphLaunch(it->second, s));
+      const bool seen = g->graphs.count(key) != 0;
+      rb_mg::Recorded* rec = nullptr;
+      RB_TRY(graph_slot(g, key, s, &rec));
+      if (seen && !rec->exec) RB_TRY(sweep_graph<VEC32>(g, cy, flexible, &rec->exec));
+      if (rec->exec) {
+        RB_CUDA(cudaGraphLaunch(rec->exec, s));
         continue;
       }
-      g->graphs.emplace(key, nullptr);
-      RB_TRY(sweep_start<VEC32>(g, cy, prm));
+      RB_TRY(sweep_start<VEC32>(g, cy));
       for (;;) {
         RB_TRY(mg_read(g, h, s));
         ++syncs;
