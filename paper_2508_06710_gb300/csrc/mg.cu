@@ -1129,6 +1129,7 @@ struct rb_mg {
   };
   std::map<std::vector<int>, Recorded> graphs;
   uint64_t launches = 0;
+  bool no_loops = false;       // the runtime did not record a loop node: sweeps stay eager
   cudaStream_t cap = nullptr;  // private stream for graph capture
 };
 
@@ -1848,7 +1849,10 @@ rb_status mg_solve_vec(rb_mg* g, const rb_cg_params& prm, const double* B, int64
       const bool seen = g->graphs.count(key) != 0;
       rb_mg::Recorded* rec = nullptr;
       RB_TRY(graph_slot(g, key, s, &rec));
-      if (seen && !rec->exec) RB_TRY(sweep_graph<VEC32>(g, cy, flexible, &rec->exec));
+      if (seen && !rec->exec && !g->no_loops) {
+        RB_TRY(sweep_graph<VEC32>(g, cy, flexible, &rec->exec));
+        g->no_loops = !rec->exec;
+      }
       if (rec->exec) {
         RB_CUDA(cudaGraphLaunch(rec->exec, s));
         continue;
