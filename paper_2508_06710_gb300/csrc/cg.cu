@@ -1188,6 +1188,7 @@ rb_status solve_vec(Solver& S_, const rb_cg_params& prm, const double* B, int64_
           // launch by launch, from a fresh direction (scale 0: k_ir_init keeps none)
           one_launch = false;
           RB_CUDA(cudaMemsetAsync(S_.sc->oscale, 0, sizeof(S_.sc->oscale), S_.s));
+          --sweep;  // a dropped sweep is none of the caller's max_sweeps
           continue;
         }
         it = (int)done;
@@ -2246,6 +2247,13 @@ bool prefer_persistent(const Solver& S_) {
          S_.n * S_.k <= 10000000;
 }
 
+// The grid barrier of a single system's launch: its limit, and arrivals beyond the grid that it waits for
+// (a build of this file for a failure-detection test sets others; a batch has rb_batch_set_barrier)
+#ifndef RB_SOLO_EXTRA_ARRIVALS
+#define RB_SOLO_EXTRA_ARRIVALS 0
+#define RB_SOLO_TIMEOUT_NS 2000000000ull
+#endif
+
 rb_status persistent_inner(Solver& S_, const rb_cg_params& prm, const Layout& L, char* base) {
   PBatch pb;
   pb.n_sys = 1;
@@ -2255,8 +2263,8 @@ rb_status persistent_inner(Solver& S_, const rb_cg_params& prm, const Layout& L,
   pb.bar = S_.sc->pbar;
   pb.err = reinterpret_cast<int*>(&S_.sc->pbar[2]);
   pb.max_iter = prm.max_iter;
-  pb.extra_arrivals = 0;
-  pb.timeout_ns = 2000000000ull;
+  pb.extra_arrivals = RB_SOLO_EXTRA_ARRIVALS;
+  pb.timeout_ns = RB_SOLO_TIMEOUT_NS;
   const bool units = units_ok(pb);
   const int grid = units ? std::min(kUGridMax, sm_count()) : std::min(kPGridMax, pcg_blocks_per_sm() * sm_count());
   partition_blocks(pb, grid, units);
