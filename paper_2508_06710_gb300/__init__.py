@@ -234,12 +234,15 @@ def _torch():
 
 def _stream(stream=None):
     """The stream's handle as an integer (what a c_void_p argument takes).  The current stream's is
-    asked for directly: the Stream object that torch.cuda.current_stream() builds costs more host
-    time (5 us) than the library's whole call."""
+    asked for directly where torch has the call (a private one): the Stream object that
+    torch.cuda.current_stream() builds costs more host time (5 us) than the library's whole call."""
     if stream is not None:
         return stream.cuda_stream
     torch = _torch()
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _ptr(t):
