@@ -67,11 +67,11 @@ std::vector<int> vec_candidates(int eb, int k) {
 //     uneven length keep the lanes, and so do few rows (24^3: too few for one lane each to hide its
 //     gathers, 27p FP32 k = 3 3.4 and in the ring 5.2).
 //   the chains in the TMA ring.  FP32, whose loads matter most, always, but for rows below 20 entries with
-//     more columns than a row has parts (27p k = 1, 3, 8 131, 153, 187 and direct 195, 221, 287; 13p k = 1,
-//     3, 8, 12 76, 83, 119, 203 and direct 88, 107, 139, 214; 27p k = 4 in halves, eight parts, 156).  FP64 is
-//     bound by its pipe: the ring for one column and 27p k = 2 in halves (13p k = 1 113 and direct 135; 27p
-//     246 and 269, k = 2 414 and 437), direct otherwise (13p k = 2, 3 193, 281 and in the ring 199, 305; 27p
-//     k = 3, 4 619, 680 and 640, 831).
+//     more columns than a row has parts (27p k = 1, 3, 4, 8 136, 146, 150, 185 and direct 195, 221, 222, 287;
+//     13p k = 1, 3, 8, 12 78, 83, 117, 199 and direct 88, 107, 139, 214).  FP64 is bound by its pipe: the
+//     ring for one column and 27p k = 2 in halves (13p k = 1 113 and direct 135; 27p 248 and 269, k = 2 408
+//     and 437), direct otherwise (13p k = 2, 3 195, 281 and in the ring 199, 305; 27p k = 3, 4 619, 680 and
+//     640, 831).
 //   grid, direct kernels.  FP64 with two columns or more: one block per row block, not a resident
 //     wave (L k = 3 91 and 97, k = 8 226 and 248, extruded k = 64 150 and 157; 27p k = 4 680 and 738); one
 //     column, the gradient's rows of two and eight chains: the wave (G k = 3 86 and 93; 27p k = 3 619 and
@@ -96,7 +96,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
   sc.stage = 0;
   sc.grid_cap = -1;
   std::vector<int> order;
-  if (mid && pipelined && (f64 ? k == 2 && len >= 20.0 : k == 4 && len >= kEightSums)) order.push_back(k / 2);
+  if (mid && pipelined && f64 && k == 2 && len >= 20.0) order.push_back(1);
   // (up to 32 columns: beyond, unaligned rows are refused, and four doubles need no alignment)
   if (csr && f64 && k % 4 == 0 && (k & (k - 1)) == 0 && k <= 32 && len < 12.0) order.push_back(4);
   if (many) order.push_back(4);

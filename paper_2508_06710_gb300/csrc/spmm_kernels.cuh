@@ -105,7 +105,7 @@ rb_status launch_csr(const rb_op* op, const SpmmSched& sc, const T* X, int64_t l
         if constexpr (sizeof(T) == 4 && VEC <= 2)
           if (op->avg_row_len >= 13.0 && op->avg_row_len < kEightSums && (sc.kp == 1 || sc.kp >= 8))
             return go(&k_spmm_tma<T, VEC, EPI, 13>, rows, cap, smem, consumers + 32);
-        if constexpr (VEC < 4)
+        if constexpr (VEC < 4 || sizeof(T) == 4)
           if (k <= 4 && op->avg_row_len >= kEightSums)
             return go(&k_spmm_tma<T, VEC, EPI, 8>, rows, cap, smem, consumers + 32);
         return go(&k_spmm_tma<T, VEC, EPI, 4>, rows, cap, smem, consumers + 32);

@@ -24,12 +24,13 @@ namespace rb {
 // rows (LONG): a tile is tens of KB, so two stages and as many consumers as keep a tile near 28 KB
 // (four blocks per SM), and each lane issues kLongGathers gathers before it uses the first: a row's
 // gathers are an L2 round trip each, and two at a time left the 16 resident consumer warps waiting.  A
-// row's sum has the parts that lanes would make of it (spmm_impl.cuh): eight, four above four columns
-// or with four columns a lane.  27-point operator, FP32 k = 8, 150^3: 187 us (957 MB: 0.76 of the measured
-// HBM rate), error against 64 bits 6.25e-8, as with the row split over four lanes (292 us); in two running
-// chains 8.3e-8.  FP64 k = 1: 246 us and 1.06e-16 (one chain 206 and 1.75e-16, eight lanes 482 and 1.06e-16).
-// Three stages, two gathers at a time or two blocks per SM all took longer (k = 8, 160^3: 347, over 380 and
-// 254 us where this shape took 216).
+// row's sum has the parts that lanes would make of it (spmm_impl.cuh): eight, or four above four columns,
+// with four FP64 columns a lane and below 16 entries.  27-point operator, FP32 k = 8, 160^3: 213 us (1.16 GB:
+// 0.81 of the measured HBM rate), error against 64 bits 6.25e-8 at 36^3, as with the row split over four
+// lanes (353 us); in two running chains 8.3e-8.  FP64 k = 1, 150^3: 248 us and 1.06e-16 (one chain 206 and
+// 1.75e-16, eight lanes 482 and 1.06e-16).  Three stages, two gathers at a time or two blocks per SM all
+// took longer (k = 8, 160^3: 347, over 380 and 254 us); with eight chains, whose registers three blocks
+// of 288 threads cramp, blocks have 160 threads (k = 3: 154 -> 146 us without that limit).
 template <bool LONG>
 constexpr int kTmaStages = LONG ? 2 : 3;
 template <typename T, int VEC, int CH>
@@ -83,7 +84,7 @@ inline int tma_capacity(const rb_op* op, int R, size_t limit) {
 
 // CH: 0 the short-row shape, otherwise the long-row one with CH partial sums a row
 template <typename T, int VEC, int EPI, int CH>
-__global__ void __launch_bounds__(kTmaThreads, CH ? (sizeof(T) == 4 ? 3 : 2) : 0)
+__global__ void __launch_bounds__(kTmaThreads, CH ? (sizeof(T) == 4 && CH != 8 ? 3 : 2) : 0)
     k_spmm_tma(CsrArgs<T> a, int R, int cap, int* __restrict__ err) {
   constexpr bool LONG = CH > 0;
   extern __shared__ __align__(128) unsigned char sm[];
