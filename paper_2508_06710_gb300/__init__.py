@@ -239,10 +239,10 @@ def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
     torch = _torch()
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    if raw is None:
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    except AttributeError:
         return torch.cuda.current_stream().cuda_stream
-    return raw(torch.cuda.current_device())
 
 
 def _ptr(t):
@@ -448,6 +448,8 @@ class Operator:
         return X, k, ldx, Y, ldy
 
     def spmm(self, X, Y=None, c=None, stream=None):
+        """Y = A X, each column scaled by c (rb_spmm).  check() reports a pipelined kernel that gave up
+        a bounded wait; the default schedule takes one for some shapes (see rb_spmm)."""
         torch = _torch()
         if Y is None:
             shape = (self.n_rows, X.shape[1], 2) if self.dtype == "df64" else (self.n_rows, X.shape[1] if X.dim() > 1 else 1)
