@@ -272,7 +272,11 @@ rb_status rb_operator_check(rb_op_t op, rb_stream_t stream);
  * DEVICE values or NULL (= 1).  For an extruded operator k must equal extruded_nz and
  * the full L3D is applied (c is then applied to the whole row).  X and Y must not
  * overlap.  Vector width, rows per block and lanes per row are chosen per (operator, k)
- * from the tuning table (rb_tune_spmm). */
+ * from the tuning table (rb_tune_spmm), by a measured rule without an entry there.  That rule
+ * takes the pipelined kernel (stage 2 below) for FP32 rows of two or many columns of a matrix
+ * beyond L2, and for even rows of 12 to 40 entries (FP32; FP64 one or two columns): a bounded
+ * wait of it that gives up leaves rows of Y unwritten with RB_OK here, and is reported by
+ * rb_operator_check. */
 rb_status rb_spmm(rb_op_t A, const void* X, int64_t ldx, void* Y, int64_t ldy, int32_t k, const double* c,
                   rb_stream_t stream);
 
@@ -290,11 +294,15 @@ rb_status rb_tune_spmm(rb_op_t A, const void* X, int64_t ldx, void* Y, int64_t l
 
 /* Schedule of the SpMM kernels for k columns (what rb_tune_spmm chooses among):
  *   vec      columns per thread (1, 2, 3 or 4; 8- and 16-byte groups are vector accesses)
- *   lpr      lanes sharing one row's nonzeros (1, 2, 4, 8), reduced with warp shuffles
+ *   lpr      parts of a row's sum (1, 2, 4, 8): lanes sharing its nonzeros, reduced with warp
+ *            shuffles, or (even rows of 12 to 40 entries, more than 24000 of them, stage 0, no
+ *            row blocks) chains of one lane, added in the same order: the same result bit for bit
  *   stage    0: indices and values read by the row's lanes directly; 1: a block's nonzeros
  *            staged in shared memory by its threads; 2: a producer warp streams each tile's
- *            row pointers, indices and values into a 3-stage shared-memory ring with TMA bulk
- *            copies (cp.async.bulk + mbarrier) while eight consumer warps compute
+ *            row pointers, indices and values into a shared-memory ring with TMA bulk copies
+ *            (cp.async.bulk + mbarrier) while up to eight consumer warps compute: three stages
+ *            and one sum a row, or (rows of 12 entries and more on average) two stages and a
+ *            row's sum in four or eight chains
  *   grid_cap -1: one resident wave of persistent blocks; 0: one block per row block; > 0: cap
  * rb_set_spmm_schedule pins a schedule for (A, k) (RB_EINVAL if it is not valid for A);
  * rb_get_spmm_schedule reports the one rb_spmm will use for k with the given layout. */

@@ -1620,9 +1620,9 @@ __global__ void __launch_bounds__(kPThreads) k_pcg_batch(PBatch b) {
 // registers: 52.3 against 50.2 ms on the batch below).  Channel 192 x 128 x 96, k = 3, per
 // iteration: 52 us (two kernels a step: 77), of which q = A p 21, the update 17, the two barriers
 // 9 and the column sums 5; bound by instruction issue and by L2: 20 M warp instructions (IPC 1.2),
-// 65 MB read and 57 MB written of the vectors that are not in shared memory.  The five uneven
-// systems 64^3 k = 8, 128^3 k = 1, 3 x 96 x 64 x 48 k = 3: 68.3 -> 50.6 ms.  Measured and not kept:
-// p in shared memory instead of r (104 ms on the channel against 82: r and d then move twice), plain
+// 65 MB read and 57 MB written of the vectors that are not in shared memory (with p's seven gathers
+// 258 MB read at L2; DRAM 16 MB read and 66 written).  The five uneven systems 64^3 k = 8, 128^3 k = 1,
+// 3 x 96 x 64 x 48 k = 3: 68.3 -> 50.6 ms.  Measured and not kept: p in shared memory instead of r (104 ms on the channel against 82: r and d then move twice), plain
 // loads of p through L1 (97), two to four units' loads issued together (109 to 118: fewer threads).
 constexpr int kUThreads = 768;
 constexpr int kUWarps = kUThreads / 32;

@@ -531,11 +531,11 @@ __global__ void __launch_bounds__(kConvThreads) k_conv3_row(Conv3Args a, int chu
 // 8: and a fourth, unused, under zero weights: N must be a multiple of 16).  Which plane a block
 // belongs to turns with zz, so B is kept three times, one per zz mod 3.  Plane zz - 1 is complete
 // after input plane zz; its block is read, zeroed and taken by plane zz + 2.  Each output adds its
-// 27 taps in the same order and groups as in the row kernel (dz, then dy, then dx pairs), so
-// results are equal bit for bit.  A CTA's MMAs and epilogue alternate; the CTAs of an SM overlap
-// them.  128^3, 8 to 8 channels: 85 -> 33 us a launch (8 to 16: 90 -> 57); the prediction of the four-level
-// network 854 -> 631 us.  33 us is not the MMAs' time (13) but the steps' chain of load, MMAs,
-// accumulator read and store at two to three CTAs an SM (four hold less than they cost in runs).
+// 27 taps in the same order and groups as in the row kernel (dz, then dy, then dx pairs).  A CTA's MMAs
+// and epilogue alternate; the CTAs of an SM overlap them.  128^3, 8 to 8 channels: 85 -> 33 us a launch
+// (8 to 16: 90 -> 57); the prediction of the four-level network 854 -> 631 us.  33 us is not the MMAs'
+// time (13) but the steps' chain of load, MMAs, accumulator read and store at two to three CTAs an SM
+// (four hold less than they cost in runs).
 constexpr int kPlaneRows = 4;
 template <int CB>
 constexpr int kPlaneN = CB == 8 ? 32 : 48;  // accumulator columns of a row

@@ -1722,8 +1722,8 @@ rb_status sweep_end(const rb_mg* g, const Cycle<float, VEC32>& cy) {
 // update of the next, run while columns iterate (k_mgcg_xr decides), and x += ||r|| d.  Replays of a
 // fixed number of iterations with a host check after each ran up to check_every - 1 idle cycles a
 // sweep (about 45 launches of 2 us each) and waited for the host between them. Channel k = 3:
-// 7.70 -> 7.21 ms; projection step on 128^3, m = 2: 22.9 -> 21.0 ms.  exec stays null where the runtime cannot
-// record a loop node (the caller then goes on eagerly).
+// 7.70 -> 7.21 ms; projection step on 128^3, m = 2: 22.9 -> 21.0 ms.  exec stays null where the runtime
+// cannot record a loop node (the caller then goes on eagerly).
 template <int VEC32>
 rb_status sweep_graph(rb_mg* g, const Cycle<float, VEC32>& cy, int flexible, cudaGraphExec_t* exec) {
   *exec = nullptr;
