@@ -215,9 +215,10 @@ __global__ void __launch_bounds__(kTmaThreads, CH ? (sizeof(T) == 4 && CH != 8 ?
 #pragma unroll
             for (int ee = 0; ee < VEC; ++ee) sum[ee] += part[0][ee];
           }
-          sum_in_chains<T, VEC, 4, 4, false>(
-              re - p, [&](int q) { return ldv<T, VEC>(Xc + (int64_t)s_ci[p + q] * a.ldx); },
-              [&](int q) { return s_va[p + q]; }, acc);
+          if (p < re)
+            sum_in_chains<T, VEC, 4, 4, false>(
+                re - p, [&](int q) { return ldv<T, VEC>(Xc + (int64_t)s_ci[p + q] * a.ldx); },
+                [&](int q) { return s_va[p + q]; }, acc);
 #pragma unroll
           for (int ee = 0; ee < VEC; ++ee) acc[ee] += sum[ee];
         } else if constexpr (LONG) {
