@@ -62,10 +62,10 @@ std::vector<int> vec_candidates(int eb, int k) {
 // the extruded mesh):
 //   long rows (12 entries on).  A row's sum has up to eight parts, fewer with more columns: eight lanes
 //     split the row while each still has a few chunks.  Where the rows are of like length, 12 to 40
-//     entries and enough of them (rows_by_chains), the parts are chains of one lane: the same sums
-//     without the shuffles (eight lanes took 13p FP64 k = 1, 3 375 and 935, 27p 482 and 1236).  Rows of
-//     uneven length keep the lanes, and so do few rows (24^3: too few for one lane each to hide its
-//     gathers, 27p FP32 k = 3 3.4 and in the ring 5.2).
+//     entries and enough of them (rows_by_chains), the parts are chains of one lane: the
+//     same sums without the shuffles (eight lanes took 13p FP64 k = 1, 3 375 and 935, 27p 482 and 1236).
+//     Rows of uneven length keep the lanes, and so do few rows (24^3: too few for one lane each to hide
+//     its gathers, 27p FP32 k = 3 3.4 and in the ring 5.2).
 //   the chains in the TMA ring.  FP32, whose loads matter most, always, but for rows below 20 entries with
 //     more columns than a row has parts (27p k = 1, 3, 4, 8 136, 146, 150, 185 and direct 195, 221, 222, 287;
 //     13p k = 1, 3, 8, 12 78, 83, 117, 199 and direct 88, 107, 139, 214).  FP64 is bound by its pipe: the
@@ -77,9 +77,11 @@ std::vector<int> vec_candidates(int eb, int k) {
 //     column, the gradient's rows of two and eight chains: the wave (G k = 3 86 and 93; 27p k = 3 619 and
 //     641).  FP32 and rows split over lanes: the wave.
 //   width.  FP64 k = 4, 8, 16, 32 on short rows: four doubles a thread (G k = 4 107 and 115, the
-//     divergence k = 8 191 and 224 with the grid).
+//     divergence k = 8 191 and 224 with the grid), on rows of two up to 16 (G k = 32 879 and 851).
 //   the TMA ring on short rows.  FP32, a matrix that does not stay in L2, and little work per entry
-//     loaded (rows of two: G k = 3 49 and 58) or many columns (L k = 16 88 and 99).
+//     loaded (rows of two: G k = 3 49 and 58) or many columns, up to 32, that use three quarters of the
+//     chunks laid out (L k = 12, 16, 24, 32 82, 87, 170, 160 and 92, 99, 176, 180; but k = 20, 48 178, 395 and
+//     170, 327).
 // The ring is taken only where every tile fits its stages (no row far above the average).
 // (`pipelined` false: a caller with kernels of its own, whose rows are read directly.)
 SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const void* X, const void* Y,
@@ -90,7 +92,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
   const double len = op->avg_row_len;
   const bool even = op->max_row_len <= 1.25 * len + 1.0;  // every tile within the ring's capacity
   const bool mid = rows_by_chains(op);
-  const bool many = csr && f32 && k >= 12 && k % 4 == 0 && len < 12.0;
+  const bool many = csr && f32 && k >= 12 && k <= 32 && k % 4 == 0 && 3 * next_pow2(k / 4) <= k && len < 12.0;
   SpmmSched sc;
   sc.lpr = 1;
   sc.stage = 0;
@@ -98,7 +100,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
   std::vector<int> order;
   if (mid && pipelined && f64 && k == 2 && len >= 20.0) order.push_back(1);
   // (up to 32 columns: beyond, unaligned rows are refused, and four doubles need no alignment)
-  if (csr && f64 && k % 4 == 0 && (k & (k - 1)) == 0 && k <= 32 && len < 12.0) order.push_back(4);
+  if (csr && f64 && k % 4 == 0 && (k & (k - 1)) == 0 && k <= (len < 4.0 ? 16 : 32) && len < 12.0) order.push_back(4);
   if (many) order.push_back(4);
   if (k * eb == 16 || k * eb == 8) order.push_back(k);
   if (k % 3 == 0 && k <= 12) order.push_back(3);
