@@ -931,7 +931,7 @@ struct Solver {
     using I2 = std::integral_constant<int, 2>;
     using I4 = std::integral_constant<int, 4>;
     using I8 = std::integral_constant<int, 8>;
-    const bool chains = rows_by_chains(op) && !(op->dtype == RB_F32 && ss.lpr == 8 && ss.vec == 1);
+    const bool chains = rows_by_chains(op, ss.kp) && !(op->dtype == RB_F32 && ss.lpr == 8 && ss.vec == 1);
     switch (ss.lpr) {
       case 2: chains ? run(one, I1(), I2()) : run(ss, I2(), I1()); break;
       case 4: chains ? run(one, I1(), I4()) : run(ss, I4(), I1()); break;

@@ -62,7 +62,7 @@ std::vector<int> vec_candidates(int eb, int k) {
 // the extruded mesh):
 //   long rows (12 entries on).  A row's sum has up to eight parts, fewer with more columns: eight lanes
 //     split the row while each still has a few chunks.  Where the rows are of like length, 12 to 40
-//     entries and enough of them (rows_by_chains), the parts are chains of one lane: the
+//     entries and enough of them (even_long_rows, rows_by_chains), the parts are chains of one lane: the
 //     same sums without the shuffles (eight lanes took 13p FP64 k = 1, 3 375 and 935, 27p 482 and 1236).
 //     Rows of uneven length keep the lanes, and so do few rows (24^3: too few for one lane each to hide
 //     its gathers, 27p FP32 k = 3 3.4 and in the ring 5.2).
@@ -71,7 +71,7 @@ std::vector<int> vec_candidates(int eb, int k) {
 //     13p k = 1, 3, 8, 12 78, 83, 117, 199 and direct 88, 107, 139, 214).  FP64 is bound by its pipe: the
 //     ring for one column and 27p k = 2 in halves (13p k = 1 113 and direct 135; 27p 248 and 269, k = 2 408
 //     and 437), direct otherwise (13p k = 2, 3 195, 281 and in the ring 199, 305; 27p k = 3, 4 619, 680 and
-//     640, 831).
+//     640, 831), but for 27p k = 3 below 100,000 rows (34^3 13.0 in the ring, direct 17.5).
 //   grid, direct kernels.  FP64 with two columns or more: one block per row block, not a resident
 //     wave (L k = 3 91 and 97, k = 8 226 and 248, extruded k = 64 150 and 157; 27p k = 4 680 and 738); one
 //     column, the gradient's rows of two and eight chains: the wave (G k = 3 86 and 93; 27p k = 3 619 and
@@ -91,7 +91,7 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
   const bool csr = op->format == RB_CSR && op->ext_nz == 0;
   const double len = op->avg_row_len;
   const bool even = op->max_row_len <= 1.25 * len + 1.0;  // every tile within the ring's capacity
-  const bool mid = rows_by_chains(op);
+  const bool mid = even_long_rows(op);
   const bool many = csr && f32 && k >= 12 && k <= 32 && k % 4 == 0 && 3 * next_pow2(k / 4) <= k && len < 12.0;
   SpmmSched sc;
   sc.lpr = 1;
@@ -117,9 +117,9 @@ SpmmSched default_sched(const rb_op* op, int k, int64_t ldx, int64_t ldy, const 
       if (mid && len < kEightSums) t.lpr = std::min(t.lpr, 4);
       if (!sched_valid(op, t, k, ldx, ldy, X, Y)) t.lpr = 1;
     }
-    if (op->format == RB_CSR && f64 && k >= 2 && len >= 4.0 && (mid ? t.lpr < 8 : t.lpr == 1)) t.grid_cap = 0;
+    if (op->format == RB_CSR && f64 && k >= 2 && len >= 4.0 && (rows_by_chains(op, t.kp) ? t.lpr < 8 : t.lpr == 1)) t.grid_cap = 0;
     const double matrix = (double)op->nnz * (4 + eb) + 4.0 * op->n_rows;
-    const bool ring = mid ? (f32 ? t.lpr > 1 || k <= 8 || len >= 20.0 : k == 1 || (len >= 20.0 && k == 2))
+    const bool ring = mid ? (f32 ? t.lpr > 1 || k <= 8 || len >= 20.0 : k == 1 || (len >= 20.0 && (k == 2 || (k == 3 && !rows_by_chains(op, t.kp)))))
                           : csr && f32 && matrix > 100e6 && (len < 4.0 || (many && w == 4)) && op->n_rblk <= 1;
     if (ring && even && pipelined) {
       SpmmSched r = t;

@@ -157,12 +157,18 @@ __device__ __forceinline__ void extruded_epilogue(const CsrArgs<T>& a, int64_t r
   }
 }
 
-// Rows of 12 to 40 entries of like length (the 13- and 27-point operators' kind), enough of them for one
-// lane each to fill the chip: their sums' parts are chains of one lane rather than lanes.
-inline bool rows_by_chains(const rb_op* op) {
+// Many rows of 12 to 40 entries of like length (the 13- and 27-point operators' kind).
+inline bool even_long_rows(const rb_op* op) {
   const double len = op->avg_row_len;
   return op->format == RB_CSR && op->ext_nz == 0 && op->n_rblk <= 1 && (op->dtype == RB_F64 || op->dtype == RB_F32) &&
          op->n_rows > 24000 && len >= 12.0 && len < 40.0 && op->max_row_len <= 1.25 * len + 1.0;
+}
+
+// Whether the parts of such a row's sum are chains of one lane rather than lanes, read directly with kp
+// chunks a row: enough lanes to hide the longer chains' gathers (27-point FP64 k = 4, two chunks: 30^3 and
+// 34^3 10.9 and 14.6 us in chains, 9.9 and 13.4 over lanes; 40^3 18.6 and 21.1).
+inline bool rows_by_chains(const rb_op* op, int kp) {
+  return even_long_rows(op) && (op->avg_row_len < 20.0 || (int64_t)op->n_rows * kp >= 100000);
 }
 
 // A row that one lane walks sums in CH chains, entry q in chain q mod CH, which are added as a tree:

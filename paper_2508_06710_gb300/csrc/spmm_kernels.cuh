@@ -121,7 +121,7 @@ rb_status launch_csr(const rb_op* op, const SpmmSched& sc, const T* X, int64_t l
     k_spmm_csr<T, VEC, LPR, EPI><<<(unsigned)std::min<int64_t>(grid, INT32_MAX), kThreads, smem, s>>>(a);
   } else {
     if constexpr (LPR > 1 && (EPI & kEpiExt) == 0) {
-      if (rows_by_chains(op)) {
+      if (rows_by_chains(op, sc.kp)) {
         auto* kern = &k_spmm_chains<T, VEC, LPR, EPI>;
         const int rows = kThreads / sc.kp;
         grid = ((int64_t)op->n_rows + rows - 1) / rows;
