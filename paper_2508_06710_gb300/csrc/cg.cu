@@ -2241,8 +2241,14 @@ void solve_tail(Solver& S_, const rb_cg_params& prm, const double* B, int64_t ld
 // step: channel 192 x 128 x 96 k = 3 (7.1 M) 52 / 77 us, 128^3 k = 4 (8.4 M) 67 / 86, 128^3 k = 1
 // 25 / 33, 45 x 64 x 31 k = 1 (one float a unit) 16 / 19, 32^3 k = 1 21 / 27; beyond, the vectors
 // stream from HBM either way and one block per SM keeps fewer loads in flight: 192 x 192 x 160
-// k = 3 (17.7 M) 164 / 160, the channel at k = 16 (37.7 M) 343 / 286.
+// k = 3 (17.7 M) 164 / 160, the channel at k = 16 (37.7 M) 343 / 286.  A launch also spares a sweep its
+// host checks, so short solves gain most; few cells along a long axis iterate long, and with two or three
+// columns a step of the small launch (22 us, at k = 1 and 4 17) takes longer than two kernels (20): k = 2, 3
+// 128 x 8 x 8 7.6, 8.6 ms against 6.8, 7.5, 256 x 16 x 8 16.5, 17.5 / 15.0, 15.5, 96 x 12 x 10 6.2, 7.0 / 5.9,
+// 6.4; but 64 x 16 x 16 3.9, 4.4 / 4.2, 4.4 and 300 x 20 x 20 17.0, 19.1 / 19.9, 21.7.
 bool prefer_persistent(const Solver& S_) {
+  const int* n = S_.A32->st_n;
+  if ((S_.k == 2 || S_.k == 3) && S_.n <= 40000 && std::max({n[0], n[1], n[2]}) >= 96) return false;
   return S_.A32->format == RB_STENCIL && unit7_table_fits(S_.A32->st_n) && unit7_width(S_.A32->st_n, S_.k) != 0 &&
          S_.n * S_.k <= 10000000;
 }
