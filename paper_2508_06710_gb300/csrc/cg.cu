@@ -2049,16 +2049,22 @@ void partition_blocks(PBatch& pb, int grid, bool units) {
 // Shared memory of k_pcg_units a block may use beside its static part (one block per SM)
 constexpr size_t kUSmem = 188 * 1024;
 
-// Whether every system takes the unit kernel; then fills their unit fields for `grid` blocks
-// (the partition must be made)
+// Whether the systems take the unit kernel: all matrix-free, and together no more floats a vector than
+// 20 M.  Beyond, one block per SM streams the vectors with fewer loads in flight than the two of
+// k_pcg_batch (two channels 192 x 128 x 96 k = 4 (18.9 M) 283 and 283 ms, k = 8 (37.7 M) 564 and 517; two 96^3
+// k = 16 (28.3 M) 122 and 116; 200^3 k = 2 (16 M) 138 and 167).
 bool units_ok(const PBatch& pb) {
-  for (int i = 0; i < pb.n_sys; ++i)
+  int64_t floats = 0;
+  for (int i = 0; i < pb.n_sys; ++i) {
     if (!pb.sys[i].mf || !unit7_table_fits(pb.sys[i].st.n) || unit7_width(pb.sys[i].st.n, pb.sys[i].k) == 0 ||
         pb.sys[i].n == 0)
       return false;
-  return pb.n_sys > 0;
+    floats += (int64_t)pb.sys[i].n * pb.sys[i].k;
+  }
+  return pb.n_sys > 0 && floats <= 20000000;
 }
 
+// The systems' unit fields (the partition must be made)
 void fill_units(PBatch& pb) {
   for (int i = 0; i < pb.n_sys; ++i) {
     PSys& S = pb.sys[i];
