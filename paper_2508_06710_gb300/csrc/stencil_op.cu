@@ -65,15 +65,17 @@ __global__ void __launch_bounds__(kThreads) k_spmm_stencil7_run(Stencil7<T> st, 
 // tabulated when the operator is made, with its scale:
 //   line: a = s w_y w_z, b_ym, b_yp = s w_z / d_y, b_zm, b_zp = s w_y / d_z, S = -(b_ym + ... + b_zp)
 //   cell: 1 / d_x below and above, their negated sum D, w_x
-// y = a (x_- / d + x_+ / d + D x_0) + w_x (b . x_yz + S x_0): ten operations a value and none per cell;
-// forming entries and diagonal from the axis tables took 14 a cell and 8 a value.  Each bracket cancels by
-// itself, so its rounding stays small: against extended precision 0.7 to 1.25e-16 (2-norm, random values)
-// and 0.45 to 0.7e-16 of |A| |x| (smooth ones), rows of seven entries 1.3 to 1.6e-16 and 0.85 to 1.0e-16.
-// (Three columns and more with the seven entries formed from the tables, 8 operations a cell and 7 a value,
-// took 121 us at k = 3, with up to 3% more error than before; with four entries and the diagonal, 28
-// operations at k = 3, 117 us, and no gain on smooth values.)  190 x 127 x 95 (one cell per thread before),
-// k = 3: 162 -> 124 us (the pipe alone: 110); 192 x 128 x 96 (runs of four cells before), k = 1, 2, 3, 4, 8: 97,
-// 131, 169, 250, 490 -> 46, 86, 127, 168, 332 us.
+// One or two columns per thread: y = a (x_- / d + x_+ / d + D x_0) + w_x (b . x_yz + S x_0), ten
+// operations a value and none per cell.  More columns: the x entries and the diagonal formed first (four
+// operations a cell), then y = c_- x_- + c_+ x_+ + diag x_0 + w_x (b . x_yz), eight a value.  Forming entries
+// and diagonal from the axis tables took 14 a cell and 8 a value.  The diagonal is minus the sum of the
+// rounded x entries and of w_x S, S rounded once; the centre's term, the largest, meets only part of the
+// others.  So the error against extended precision is 0.7 to 1.25e-16 (2-norm, random values) and 0.45 to
+// 0.9e-16 of |A| |x| (smooth ones), where rows of seven entries have 1.3 to 1.6e-16 and 0.85 to 1.1e-16.
+// (Seven entries formed from the tables, 8 operations a cell and 7 a value, took 121 us at k = 3 with up to
+// 3% more error than such rows; the two brackets at every width 124.)  190 x 127 x 95 (one cell per thread
+// before), k = 3: 162 -> 116 us (the pipe alone: 103); 192 x 128 x 96 (runs of four cells before), k = 1, 2, 3, 4,
+// 8: 97, 131, 169, 250, 490 -> 46, 86, 119, 168, 332 us.
 struct alignas(16) LineCoef {
   double a, bym, byp, bzm, bzp, s;
 };
@@ -111,15 +113,28 @@ __global__ void __launch_bounds__(kThreads) k_spmm_stencil7_f64(Stencil7<double>
     const CellCoef t = cells[i];
     const LineCoef l = lines[line];
     Vec<double, VEC> y;
+    if constexpr (VEC <= 2) {
 #pragma unroll
-    for (int q = 0; q < VEC; ++q) {
-      const double u = fma(t.d, x0.v[q], fma(t.p, xp.v[q], t.m * xm.v[q]));
-      double v = l.s * x0.v[q];
-      v = fma(l.bym, ym.v[q], v);
-      v = fma(l.byp, yp.v[q], v);
-      v = fma(l.bzm, um.v[q], v);
-      v = fma(l.bzp, up.v[q], v);
-      y.v[q] = fma(l.a, u, t.w * v);
+      for (int q = 0; q < VEC; ++q) {
+        const double u = fma(t.d, x0.v[q], fma(t.p, xp.v[q], t.m * xm.v[q]));
+        double v = l.s * x0.v[q];
+        v = fma(l.bym, ym.v[q], v);
+        v = fma(l.byp, yp.v[q], v);
+        v = fma(l.bzm, um.v[q], v);
+        v = fma(l.bzp, up.v[q], v);
+        y.v[q] = fma(l.a, u, t.w * v);
+      }
+    } else {
+      const double cxm = l.a * t.m, cxp = l.a * t.p, diag = fma(t.w, l.s, -(cxm + cxp));
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) {
+        const double u = fma(diag, x0.v[q], fma(cxp, xp.v[q], cxm * xm.v[q]));
+        double v = l.bzm * um.v[q];
+        v = fma(l.bzp, up.v[q], v);
+        v = fma(l.bym, ym.v[q], v);
+        v = fma(l.byp, yp.v[q], v);
+        y.v[q] = fma(t.w, v, u);
+      }
     }
     if constexpr (SCALE) {
 #pragma unroll
