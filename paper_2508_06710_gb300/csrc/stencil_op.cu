@@ -70,8 +70,9 @@ __global__ void __launch_bounds__(kThreads) k_spmm_stencil7_run(Stencil7<T> st, 
 // operations a cell), then y = c_- x_- + c_+ x_+ + diag x_0 + w_x (b . x_yz), eight a value.  Forming entries
 // and diagonal from the axis tables took 14 a cell and 8 a value.  The diagonal is minus the sum of the
 // rounded x entries and of w_x S, S rounded once; the centre's term, the largest, meets only part of the
-// others.  So the error against extended precision is 0.7 to 1.25e-16 (2-norm, random values) and 0.45 to
-// 0.9e-16 of |A| |x| (smooth ones), where rows of seven entries have 1.3 to 1.6e-16 and 0.85 to 1.1e-16.
+// others.  So the error against extended precision is 0.7 to 1.45e-16 (2-norm, random values) and 0.45 to
+// 0.9e-16 of |A| |x| (smooth ones), on each grid below that of rows of seven entries (1.3 to 1.65e-16 and
+// 0.85 to 1.05e-16).
 // (Seven entries formed from the tables, 8 operations a cell and 7 a value, took 121 us at k = 3 with up to
 // 3% more error than such rows; the two brackets at every width 124.)  190 x 127 x 95 (one cell per thread
 // before), k = 3: 162 -> 116 us (the pipe alone: 103); 192 x 128 x 96 (runs of four cells before), k = 1, 2, 3, 4,
